@@ -37,12 +37,29 @@ struct Num<float> {
     q = small ? p : 1.0f - ex;
     e = small ? 1.0f - p : ex;
   }
+  // the two halves of absorb_pair for the stepping loop: whether a segment
+  // is thin, and q, e from x and, for a thick one, ex = exp(-x)
+  static __device__ __forceinline__ bool thin_seg(float x) { return x < 0.125f; }
+  static __device__ __forceinline__ void absorb_given(float x, float ex, float& q, float& e) {
+    const float p = x * (1.0f - x * (0.5f - x * (1.0f / 6.0f - x * (1.0f / 24.0f - x * (1.0f / 120.0f - x * (1.0f / 720.0f))))));
+    const bool small = thin_seg(x);
+    q = small ? p : 1.0f - ex;
+    e = small ? 1.0f - p : ex;
+  }
   static __device__ __forceinline__ float exp_(float x) { return expf(x); }
   static __device__ __forceinline__ float sqrt_(float x) { return sqrtf(x); }
   static __device__ __forceinline__ float floor_(float x) { return floorf(x); }
   static __device__ __forceinline__ float ldexp_(float x, int e) { return ldexpf(x, e); }
   static __device__ __forceinline__ void sincos2pi(float u, float* s, float* c) { sincospif(2.0f * u, s, c); }
   static __device__ __forceinline__ float inf() { return CUDART_INF_F; }
+  // 1 for d > 0, else 0: the offset of the face ahead.  A saturated multiply,
+  // so that the stepping loop's selects stay off the integer/compare pipe
+  // (a component below 1e-38 has an infinite reciprocal: its face is never
+  // the nearest, whatever comes out here)
+  static __device__ __forceinline__ float ahead(float d) { return __saturatef(d * 3.0e38f); }
+  // offset f moved by t along d, kept in [0, 1]
+  static __device__ __forceinline__ float moved01(float f, float t, float d) { return __saturatef(fmaf(t, d, f)); }
+  static __device__ __forceinline__ float min_(float a, float b) { return fminf(a, b); }
   // 2^-l for 0 <= l <= 126, exact
   static __device__ __forceinline__ float pow2m(int l) { return __int_as_float((127 - l) << 23); }
   static __device__ __forceinline__ float leaf_rho(uint32_t w, double) { return __uint_as_float(w); }
@@ -72,12 +89,20 @@ struct Num<double> {
       q = 1.0 - e;
     }
   }
+  static __device__ __forceinline__ bool thin_seg(double) { return true; }
+  static __device__ __forceinline__ void absorb_given(double x, double, double& q, double& e) { absorb_pair(x, q, e); }
   static __device__ __forceinline__ double exp_(double x) { return exp(x); }
   static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
   static __device__ __forceinline__ double floor_(double x) { return floor(x); }
   static __device__ __forceinline__ double ldexp_(double x, int e) { return ldexp(x, e); }
   static __device__ __forceinline__ void sincos2pi(double u, double* s, double* c) { sincospi(2.0 * u, s, c); }
   static __device__ __forceinline__ double inf() { return CUDART_INF; }
+  static __device__ __forceinline__ double ahead(double d) { return d > 0.0 ? 1.0 : 0.0; }
+  static __device__ __forceinline__ double moved01(double f, double t, double d) {
+    const double v = fma(t, d, f);
+    return v < 0.0 ? 0.0 : (v > 1.0 ? 1.0 : v);
+  }
+  static __device__ __forceinline__ double min_(double a, double b) { return fmin(a, b); }
   static __device__ __forceinline__ double pow2m(int l) { return __longlong_as_double((long long)(1023 - l) << 52); }
   static __device__ __forceinline__ double leaf_rho(uint32_t, double r64) { return r64; }
   static __device__ __forceinline__ double load_rho64(const double* p, uint32_t i) { return __ldg(p + i); }
@@ -339,6 +364,70 @@ __device__ __forceinline__ bool advance_axis(const GridRegs& G, Geo<R>& g, Curso
   g.cz = (!a0 && !a1) ? cnew : g.cz;
   const bool inside = (cnew >> g.lev) < (a0 ? G.rx : (a1 ? G.ry : G.rz));
   neighbour_start(G, g.lev, g.idx, g.cx, g.cy, g.cz, a, plus, cold ^ cnew, P, cur);
+  return inside;
+}
+
+// The face a package leaves its leaf through: exit distance t (leaf-local
+// units; ties -> lowest axis; a component d == 0 gives NaN or inf and is
+// never selected) and its axis as two flags (x, else y, else z).  s is 1 on
+// the axes the package moves up on, else 0.  The distance to the face ahead
+// is |s - f|, and the axis follows from the minimum: no selects.
+template <typename R>
+struct Exit {
+  R t, sx, sy, sz;
+  bool x, y;
+};
+template <typename R>
+__device__ __forceinline__ Exit<R> exit_face(const Geo<R>& g, R dx, R dy, R dz, R ix, R iy, R iz) {
+  Exit<R> E;
+  E.sx = Num<R>::ahead(dx);
+  E.sy = Num<R>::ahead(dy);
+  E.sz = Num<R>::ahead(dz);
+  const R tx = fabs(E.sx - g.fx) * ix, ty = fabs(E.sy - g.fy) * iy, tz = fabs(E.sz - g.fz) * iz;
+  E.t = Num<R>::min_(Num<R>::min_(tx, ty), tz);
+  E.x = tx == E.t;
+  E.y = !E.x && ty == E.t;
+  return E;
+}
+
+// Move by t from leaf idx and, with go, cross that face (as advance(), which
+// takes the axis as a number): the offsets move and stay in [0, 1], the
+// offset on the crossing axis becomes that of the neighbour's near face, the
+// cursor aims at the neighbour.  Without go the cursor and the lattice
+// coordinates stay.  False when the package leaves the root grid.
+template <typename R>
+__device__ __forceinline__ bool cross_face(const GridRegs& G, Geo<R>& g, Cursor& cur, uint32_t idx, const Exit<R>& E,
+                                           R t, bool go, R dx, R dy, R dz, uint32_t& moved, AncPath& P) {
+  const bool ex = go && E.x, ey = go && E.y, ez = go && !E.x && !E.y;
+  const R nx = Num<R>::moved01(g.fx, t, dx), ny = Num<R>::moved01(g.fy, t, dy), nz = Num<R>::moved01(g.fz, t, dz);
+  const R sa = ex ? E.sx : (ey ? E.sy : E.sz);
+  const R fnew = R(1) - sa;
+  g.fx = ex ? fnew : nx;
+  g.fy = ey ? fnew : ny;
+  g.fz = ez ? fnew : nz;
+  const uint32_t sgn = sa > R(0) ? 1u : 0xFFFFFFFFu;
+  const uint32_t cold = ex ? g.cx : (ey ? g.cy : g.cz);
+  const uint32_t cnew = cold + sgn;
+  g.cx = ex ? cnew : g.cx;
+  g.cy = ey ? cnew : g.cy;
+  g.cz = ez ? cnew : g.cz;
+  moved = cold ^ cnew;
+  const bool inside = (cnew >> g.lev) < (ex ? G.rx : (ey ? G.ry : G.rz));
+  const bool root_level = g.lev == 0;
+  const bool near = root_level || moved < 2u || !go;  // root-level neighbour or sibling: one load
+  const uint32_t sib = ex ? 1u : (ey ? 2u : 4u);
+  const uint32_t root = (g.cx >> g.lev) + G.rx * ((g.cy >> g.lev) + G.ry * (g.cz >> g.lev));
+  if (P.cap > 0 && !near) {
+    const int m = g.lev - (31 - __clz((int)moved));
+    const bool up = m >= 1 && m < P.n;
+    cur.pending = up ? P.a[m * P.stride] + sgn * sib : root;
+    cur.k = up ? m : 0;
+    P.n = up ? P.n : P.cap;
+  } else {
+    const uint32_t step = root_level ? (ex ? 1u : (ey ? G.rx : G.rx * G.ry)) : sib;
+    cur.pending = near ? idx + (go ? sgn * step : 0u) : root;
+    cur.k = near ? g.lev : 0;
+  }
   return inside;
 }
 

@@ -138,9 +138,45 @@ struct SlotNum<double> {
   static __device__ __forceinline__ double value(unsigned long long q, int) { return __longlong_as_double((long long)q); }
 };
 
+// Sum of a fixed-point energy / a count over the lanes of mask m, exact: the
+// value is summed in limbs narrow enough that 32 of them fit one 32-bit
+// warp reduction.
+__device__ __forceinline__ unsigned long long sum_lanes_u64(unsigned m, unsigned long long q) {
+  const unsigned a = __reduce_add_sync(m, (unsigned)q & 0x3FFFFFu);
+  const unsigned b = __reduce_add_sync(m, (unsigned)(q >> 22) & 0x3FFFFFu);
+  const unsigned c = __reduce_add_sync(m, (unsigned)(q >> 44));
+  return (unsigned long long)a + ((unsigned long long)b << 22) + ((unsigned long long)c << 44);
+}
+__device__ __forceinline__ unsigned long long sum_lanes_u32(unsigned m, uint32_t v) {
+  const unsigned a = __reduce_add_sync(m, v & 0xFFFFu), b = __reduce_add_sync(m, v >> 16);
+  return (unsigned long long)a + ((unsigned long long)b << 16);
+}
+
+// The slot of the job that all calling lanes (mask m) book to; -1: they book
+// to several jobs, or to one without a slot.
+__device__ __forceinline__ int common_slot(const WarpLedger& SL, unsigned m, int job, int wid) {
+  const int j0 = __shfl_sync(m, job, __ffs(m) - 1);
+  const bool same = __all_sync(m, job == j0);
+  if (!same) return -1;
+  return SL.tag[0][wid] == j0 ? 0 : (SL.tag[1][wid] == j0 ? 1 : -1);
+}
+
+// Bookings come in batches: the lanes that book together are summed in
+// registers and one of them updates the slot.  (A 64-bit atomic add to
+// shared memory is a compare-and-swap loop, which 8 to 32 lanes adding to
+// one address run 8 to 32 times.)
 template <typename R>
 __device__ __forceinline__ void book_d(WarpLedger& SL, const JobDev* jobs, int job, int wid, int i, R v) {
   if (v == R(0)) return;
+  if (sizeof(R) == 4) {
+    const unsigned m = __activemask();
+    const int sl = common_slot(SL, m, job, wid);
+    if (sl >= 0) {
+      const unsigned long long q = sum_lanes_u64(m, to_fixed((float)v, SL.shift[sl][wid]));
+      if ((threadIdx.x & 31) == (unsigned)(__ffs(m) - 1)) atomicAdd(&SL.d[sl][i][wid], q);
+      return;
+    }
+  }
   if (SL.tag[0][wid] == job) {
     SlotNum<R>::add(&SL.d[0][i][wid], v, SL.shift[0][wid]);
   } else if (SL.tag[1][wid] == job) {
@@ -150,15 +186,19 @@ __device__ __forceinline__ void book_d(WarpLedger& SL, const JobDev* jobs, int j
   }
 }
 
-__device__ __forceinline__ void book_u(WarpLedger& SL, const JobDev* jobs, int job, int wid, int i,
-                                       unsigned long long v) {
-  if (v == 0ull) return;
-  if (SL.tag[0][wid] == job) {
-    atomicAdd(&SL.u[0][i][wid], v);
+__device__ __forceinline__ void book_u(WarpLedger& SL, const JobDev* jobs, int job, int wid, int i, uint32_t v) {
+  if (v == 0u) return;
+  const unsigned m = __activemask();
+  const int sl = common_slot(SL, m, job, wid);
+  if (sl >= 0) {
+    const unsigned long long q = sum_lanes_u32(m, v);
+    if ((threadIdx.x & 31) == (unsigned)(__ffs(m) - 1)) atomicAdd(&SL.u[sl][i][wid], q);
+  } else if (SL.tag[0][wid] == job) {
+    atomicAdd(&SL.u[0][i][wid], (unsigned long long)v);
   } else if (SL.tag[1][wid] == job) {
-    atomicAdd(&SL.u[1][i][wid], v);
+    atomicAdd(&SL.u[1][i][wid], (unsigned long long)v);
   } else {
-    atomicAdd(ledger_u(jobs[job].ledger, i), v);
+    atomicAdd(ledger_u(jobs[job].ledger, i), (unsigned long long)v);
   }
 }
 
@@ -229,8 +269,16 @@ enum { EV_NONE = 0, EV_IDLE, EV_INTERACT, EV_ESCAPE, EV_CUT, EV_KILL, EV_DEGEN, 
 // waiting events together.  Each visit to the event code costs the warp the
 // same whatever the number of lanes it serves, so serving one event per
 // visit (batch 1) spends most issue slots on lanes that do nothing.
+// Batches of 8 / 10 / 12 / 16 / 20 lanes: the tiled rounds of a 256^3 cloud
+// step (4e7 packages) 180.8 / 167.8 / 158.9 / 153.4 / 156.1 ms, where most
+// events write a record; the untiled 128^3 cloud (4e6 packages) 5.17 / 5.08 /
+// 5.11 / 5.35 / 5.76 ms, a batched launch of 16 models 8.00 / 7.80 / 7.69 /
+// 7.49 / 7.80 ms.
 #ifndef RT_EV_BATCH
-#define RT_EV_BATCH 8
+#define RT_EV_BATCH 12
+#endif
+#ifndef RT_EV_BATCH_TILED
+#define RT_EV_BATCH_TILED 16
 #endif
 #ifndef RT_PEEL_EV_BATCH
 #define RT_PEEL_EV_BATCH 8
@@ -550,6 +598,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
   G.rx = G.ry = G.rz = 1u;
   R dx = R(0), dy = R(0), dz = R(1), ix = R(0), iy = R(0), iz = R(0);
   R W = R(0), tau = R(0), taup = R(0), pkt_abs = R(0), kext = R(0), alb = R(0), tau_cut = R(0);
+  R thin_lim = R(0);       // extinction per local unit below which a deposit is taken from the f64 density
   double* absb = nullptr;
   unsigned int* hitp = nullptr;
   uint32_t step_limit = 0u, ncross = 0u, npeel = 0u;
@@ -557,6 +606,14 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
   double* selfb = nullptr; // ALI: self-absorption tally (LEVELS kernels)
   int plev = -1;           // resampling: grid level of the last cell (capped), -1: none yet
   int splt_lmax = 0;       // resampling: the cap of the grid levels
+
+  // the word (and, in FP64, the density) of the node the cursor points at
+  uint32_t w = 0u;
+  double r64 = 0.0;
+  auto fetch_node = [&]() {
+    w = ld_node(G.node + cur.pending);
+    r64 = Num<R>::load_rho64(G.rho64, cur.pending);
+  };
 
   // after a scattering (and its peel-off): new direction from the phase
   // function, Russian roulette when the weight is low, next free path.
@@ -660,6 +717,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
           G.ry = J.root[1];
           G.rz = J.root[2];
           step_limit = (uint32_t)min(J.step_limit, (long long)0xFFFFFFFFll);
+          thin_lim = sizeof(R) == 4 && J.thin64 ? R(FLT_MIN) : R(0);
           tau_cut = Num<R>::tau_max(J) > R(0) ? Num<R>::tau_max(J) : Num<R>::inf();
           const long long p = gi - I.pkt_begin;
           const int bin = (int)((r.meta >> 5) & 255u);
@@ -721,6 +779,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
           cur.k = 0;
           P.n = P.cap;
           st = ST_TRACE;
+          fetch_node();
         } else {
           // ------------------------------------------------ emission (Sect. 2.3)
           const ItemDev& I = items[lo];
@@ -734,6 +793,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
           G.ry = J.root[1];
           G.rz = J.root[2];
           step_limit = (uint32_t)min(J.step_limit, (long long)0xFFFFFFFFll);
+          thin_lim = sizeof(R) == 4 && J.thin64 ? R(FLT_MIN) : R(0);
           tau_cut = Num<R>::tau_max(J) > R(0) ? Num<R>::tau_max(J) : Num<R>::inf();
           const long long p = gi - I.pkt_begin;
           int blo = 0, bhi = J.n_lambda - 1;
@@ -772,7 +832,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
           ncross = npeel = 0u;
           C.nscat[t] = 0;
           book_d(SL, jobs, job, wid, L_EMIT, W0);
-          book_u(SL, jobs, job, wid, U_PK, 1ull);
+          book_u(SL, jobs, job, wid, U_PK, 1u);
           bool inside;
           if (I.kind == RT_SRC_POINT || I.kind == RT_SRC_BEAM) {
             if (I.kind == RT_SRC_POINT) {
@@ -859,6 +919,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
           }
           if (inside) {
             st = ST_TRACE;
+            if (MODE != 1) fetch_node();
           } else {
             book_d(SL, jobs, job, wid, L_ESC, W);
             const long long li = C.log_index[t];
@@ -887,128 +948,244 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
     }
 
     // ------------------------------------------------------------- fast path
-    // Step cells until some lane of the warp meets an event.  One node word
-    // is loaded per lane per pass: a refined node advances the descent by a
-    // level, a leaf gets one segment (Sect. 2.3) and a face crossing.
+    // Step cells until RT_EV_BATCH lanes of the warp have met an event, or
+    // none steps any more.  One node word per lane and pass: a refined node
+    // advances the descent by a level, a leaf gets one segment (Sect. 2.3)
+    // and a face crossing.  The word of the next node is fetched as soon as
+    // the crossing has named it, so the segment's absorption and deposit run
+    // while the load is under way.
     int ev = (st == ST_TRACE || st == ST_PEEL) ? EV_NONE : EV_IDLE;
     // one pass of the loop; a warp none of whose lanes marches an inline
     // peel-off (the deferred queue had room) runs the tracing-only form
-    auto pass = [&](auto trace_only) {
-      constexpr bool TRACE_ONLY = decltype(trace_only)::value;
-        if (ev == EV_NONE) {
-          const uint32_t w = ld_node(G.node + cur.pending);
-          const double r64 = Num<R>::load_rho64(G.rho64, cur.pending);
-          if (w & RT_INTERIOR) {
-            descend_step(g, cur, w, dx, dy, dz, P);
-            if (RT_COUNT_DESCENTS) atomicAdd(&g_descents[(TRACE_ONLY || st == ST_TRACE) ? 0 : 1], 1ull);
+    auto pass = [&]() {
+      if (ev == EV_NONE) {
+        if (w & RT_INTERIOR) {
+          descend_step(g, cur, w, dx, dy, dz, P);
+          if (RT_COUNT_DESCENTS) atomicAdd(&g_descents[st == ST_TRACE ? 0 : 1], 1ull);
+          fetch_node();
+        } else {
+          settle_leaf(g, cur, w, r64);
+          const bool tr = st == ST_TRACE;
+          const uint32_t leaf = cur.pending;
+          const Exit<R> E = exit_face(g, dx, dy, dz, ix, iy, iz);
+          const R tx = E.t;
+          int lvs = 0;
+          if (SPLIT && tr) {
+            lvs = min(g.lev, splt_lmax);
+            if (plev < 0) plev = lvs;
+          }
+          if (tr && ncross >= step_limit) {
+            ev = EV_KILL;
+          } else if (!(tx < Num<R>::inf())) {
+            ev = EV_DEGEN;  // cannot happen for |d| = 1
+          } else if (SPLIT && tr && lvs != plev) {
+            ev = EV_SPLIT;  // entered a grid of another level: resample first
           } else {
-            settle_leaf(g, cur, w, r64);
-            const bool tr = TRACE_ONLY || st == ST_TRACE;
-            int a;
-            uint32_t moved = 0u;
-            const R tx = exit_dist(g, dx, dy, dz, ix, iy, iz, a);
-            int lvs = 0;
-            if (SPLIT && tr) {
-              lvs = min(g.lev, splt_lmax);
-              if (plev < 0) plev = lvs;
+            const int lev = g.lev;
+            const R kl = kext * g.rho * Num<R>::pow2m(lev);  // extinction per local unit
+            // continuous: the free path is drawn in scattering optical depth
+            // (the weight decays by the absorbed fraction along the segment);
+            // analog: in extinction optical depth
+            const R kev = EST == RT_EST_CONTINUOUS ? alb * kl : kl;
+            const R tev = kev * tx;
+            const bool inside_event = tr && kev > R(0) && tev >= tau;
+            R tseg = tx;
+            double* const dep_to = absb;
+            if (!tr) {
+              taup += kl * tx;
+              npeel += tx > R(0) ? 1u : 0u;
             }
-            if (tr && ncross >= step_limit) {
-              ev = EV_KILL;
-            } else if (a < 0) {
-              ev = EV_DEGEN;  // cannot happen for |d| = 1
-            } else if (SPLIT && tr && lvs != plev) {
-              ev = EV_SPLIT;  // entered a grid of another level: resample first
+            if (inside_event) {
+              tseg = tau / kev;
+              g.fx = Num<R>::moved01(g.fx, tseg, dx);
+              g.fy = Num<R>::moved01(g.fy, tseg, dy);
+              g.fz = Num<R>::moved01(g.fz, tseg, dz);
+              ev = EV_INTERACT;
+            } else if (!tr && taup > tau_cut) {
+              ev = EV_CUT;
             } else {
-              const R kl = kext * g.rho * Num<R>::pow2m(g.lev);  // extinction per local unit
-              bool inside_event = false;
-              R tseg = tx;
+              uint32_t moved;
+              const int ax = E.x ? 0 : (E.y ? 1 : 2);
+              if (!advance(G, g, cur, ax, tx, dx, dy, dz, moved, P)) {
+                ev = EV_ESCAPE;
+              } else {
+                fetch_node();
+                if (MODE == 2 && tr && (moved >> (lev + T.tsh)) != 0u) ev = EV_TILE;  // entered another tile: next round
+                // (the search for the neighbour starts at or above the level
+                // of the crossed face: cur.k <= that level)
+                if (LEVELS && tr && cur.k < mlev && crossed_grid_level(g, ax, dx, dy, dz) < mlev) {
+                  const JobDev& J = jobs[C.job[t]];
+                  const int v = crossed_grid_level(g, ax, dx, dy, dz);
+                  if (v <= J.sub_conf) {
+                    ev = EV_ESCAPE;  // left the subtree of this subiteration
+                  } else {
+                    mlev = v;
+                    absb = J.absorbed ? J.absorbed + (long long)mlev * J.n_cells : nullptr;
+                  }
+                }
+              }
+            }
+            if (tr) {
               if (EST == RT_EST_CONTINUOUS) {
-                // free path drawn in scattering optical depth; the weight
-                // decays by the absorbed fraction along the segment
-                const R ksca = alb * kl;
-                const R tsc = ksca * tx;
-                inside_event = tr && ksca > R(0) && tsc >= tau;
-                if (inside_event) tseg = tau / ksca;
-                if (tr) {
-                  R q, e;
-                  Num<R>::absorb_pair((kl - ksca) * tseg, q, e);
-                  tau = inside_event ? R(0) : tau - tsc;
-                  const R dep = W * q;
-                  W = W * e;
-                  const bool thin = sizeof(R) == 4 && !(kl >= R(FLT_MIN));
-                  if (dep > R(0) && !thin) {
-                    pkt_abs += dep;
-                    if (absb) red_acc(absb + g.idx, widen(dep));
-                    if (HITS && hitp) atomicAdd(hitp + g.idx, 1u);
-                    if (LEVELS && selfb && g.idx == orig_t) atomicAdd(selfb + g.idx, widen(dep));
-                  } else if (thin && tseg > R(0) && jobs[C.job[t]].thin64) {
-                    // a near-vacuum cell: its extinction per unit length is
-                    // below the f32 normal range, so the deposit is taken
-                    // from the f64 density in the thin limit q = x (x <
-                    // 1e-38; the weight and the free path do not change)
-                    const JobDev& J = jobs[C.job[t]];
-                    const BinDev& B = J.bins[C.bin[t]];
-                    const double x = (1.0 - B.albedo_d) * B.kext_d * __ldg(J.rho64 + g.idx) *
-                                     Num<double>::pow2m(g.lev) * (double)tseg;
-                    const double d64 = widen(W) * x;
-                    if (d64 > 0.0) {
-                      if (absb) red_acc(absb + g.idx, d64);
-                      if (HITS && hitp) atomicAdd(hitp + g.idx, 1u);
-                      if (LEVELS && selfb && g.idx == orig_t) atomicAdd(selfb + g.idx, d64);
-                    }
+                R q, e;
+                Num<R>::absorb_pair((kl - kev) * tseg, q, e);
+                tau = inside_event ? R(0) : tau - tev;
+                const R dep = W * q;
+                W = W * e;
+                const bool thin = sizeof(R) == 4 && !(kl >= R(FLT_MIN));
+                if (dep > R(0) && !thin) {
+                  pkt_abs += dep;
+                  if (dep_to) red_acc(dep_to + leaf, widen(dep));
+                  if (HITS && hitp) atomicAdd(hitp + leaf, 1u);
+                  if (LEVELS && selfb && leaf == orig_t) atomicAdd(selfb + leaf, widen(dep));
+                } else if (thin && tseg > R(0) && jobs[C.job[t]].thin64) {
+                  // a near-vacuum cell: its extinction per unit length is
+                  // below the f32 normal range, so the deposit is taken
+                  // from the f64 density in the thin limit q = x (x <
+                  // 1e-38; the weight and the free path do not change)
+                  const JobDev& J = jobs[C.job[t]];
+                  const BinDev& B = J.bins[C.bin[t]];
+                  const double x = (1.0 - B.albedo_d) * B.kext_d * __ldg(J.rho64 + leaf) * Num<double>::pow2m(lev) *
+                                   (double)tseg;
+                  const double d64 = widen(W) * x;
+                  if (d64 > 0.0) {
+                    if (dep_to) red_acc(dep_to + leaf, d64);
+                    if (HITS && hitp) atomicAdd(hitp + leaf, 1u);
+                    if (LEVELS && selfb && leaf == orig_t) atomicAdd(selfb + leaf, d64);
                   }
                 }
               } else {
-                // analog: free path drawn in extinction optical depth
-                const R te = kl * tx;
-                inside_event = tr && kl > R(0) && te >= tau;
-                if (inside_event) tseg = tau / kl;
-                if (tr) tau = inside_event ? R(0) : tau - te;
+                tau = inside_event ? R(0) : tau - tev;
               }
-              if (tr) {
-                ncross += tseg > R(0) ? 1u : 0u;
-              } else {
-                taup += kl * tx;
-                npeel += tx > R(0) ? 1u : 0u;
-              }
-              if (inside_event) {
-                g.fx = clamp01(g.fx + tseg * dx);
-                g.fy = clamp01(g.fy + tseg * dy);
-                g.fz = clamp01(g.fz + tseg * dz);
-                cur.pending = g.idx;
-                cur.k = g.lev;
-                ev = EV_INTERACT;
-              } else if (!tr && taup > tau_cut) {
-                ev = EV_CUT;
-              } else if (!advance(G, g, cur, a, tx, dx, dy, dz, moved, P)) {
-                ev = EV_ESCAPE;
-              } else if (LEVELS && tr && cur.k < mlev && crossed_grid_level(g, a, dx, dy, dz) < mlev) {
-                // (the search for the neighbour starts at or above the level
-                // of the crossed face: cur.k <= that level)
-                const JobDev& J = jobs[C.job[t]];
-                const int v = crossed_grid_level(g, a, dx, dy, dz);
-                if (v <= J.sub_conf) {
-                  ev = EV_ESCAPE;  // left the subtree of this subiteration
-                } else {
-                  mlev = v;
-                  absb = J.absorbed ? J.absorbed + (long long)mlev * J.n_cells : nullptr;
-                  if (MODE == 2 && (moved >> (g.lev + T.tsh)) != 0u) ev = EV_TILE;
-                }
-              } else if (MODE == 2 && tr && (moved >> (g.lev + T.tsh)) != 0u) {
-                ev = EV_TILE;  // entered another tile: next round
-              }
+              ncross += tseg > R(0) ? 1u : 0u;
             }
           }
         }
+      }
     };
+    // The tracing-only pass.  On large grids it is bound by the SM's random
+    // accesses: one 4-byte load and one FP64 reduction per crossing to cells
+    // in the L2 run at 1.2e11 per second at most (a kernel that does nothing
+    // else; 2.9e11 loads or 2.0e11 reductions alone), and the untiled 128^3
+    // cloud reaches 1.15e11.  On grids of 1e5..1e6 cells it is bound by the
+    // length of its dependent chain, so everything a common segment needs is
+    // straight-line; what few lanes need (a refined node, a leaf coarser than
+    // the lattice level, the step limit) takes the pass for itself, and one
+    // more branch holds what few segments need (an interaction inside the
+    // segment, a thick segment's exponential, a near-vacuum deposit).  The
+    // crossing comes before the segment's deposit, so that the word of the
+    // next node is under way meanwhile (7e5 cells, 2.1e6 packages: 2.42 ms ->
+    // 2.24 ms; the deposit first: 2.31 ms; fetching a whole pass ahead, with
+    // the registers that takes: 2.44 to 2.55 ms).
+    auto pass_trace = [&]() {
+      if (ev != EV_NONE) return;
+      if ((w & RT_INTERIOR) || cur.k < g.lev || ncross >= step_limit) {
+        if (w & RT_INTERIOR) {
+          descend_step(g, cur, w, dx, dy, dz, P);
+          if (RT_COUNT_DESCENTS) atomicAdd(&g_descents[0], 1ull);
+          fetch_node();
+          return;
+        }
+        if (cur.k < g.lev) settle_leaf(g, cur, w, r64);
+        if (ncross >= step_limit) ev = EV_KILL;
+        return;
+      }
+      const uint32_t leaf = cur.pending;
+      const int lev = g.lev;
+      if (SPLIT) {
+        const int lvs = min(lev, splt_lmax);
+        if (plev < 0) plev = lvs;
+        if (lvs != plev) {
+          ev = EV_SPLIT;  // entered a grid of another level: resample first
+          return;
+        }
+      }
+      const Exit<R> E = exit_face(g, dx, dy, dz, ix, iy, iz);
+      const R kl = kext * Num<R>::leaf_rho(w, r64) * Num<R>::pow2m(lev);  // extinction per local unit
+      // continuous: the free path is drawn in scattering optical depth (the
+      // weight decays by the absorbed fraction along the segment); analog:
+      // in extinction optical depth.  tau > 0, so an interaction has kev > 0
+      const R kev = EST == RT_EST_CONTINUOUS ? alb * kl : kl;
+      const R tev = kev * E.t;
+      const bool hit = tev >= tau;
+      double* const dep_to = absb;
+      R tseg = E.t, x = R(0), ex = R(1);
+      if (EST == RT_EST_CONTINUOUS) {
+        const R ka = kl - kev;
+        x = ka * tseg;
+        if (hit || !Num<R>::thin_seg(x) || !(kl >= thin_lim)) {
+          if (hit) {
+            tseg = tau / kev;
+            x = ka * tseg;
+          }
+          if (!Num<R>::thin_seg(x)) ex = Num<R>::exp_(-x);
+          if (!(kl >= thin_lim) && tseg > R(0)) {
+            // a near-vacuum cell: its extinction per unit length is below
+            // the f32 normal range, so the deposit is taken from the f64
+            // density in the thin limit q = x (x < 1e-38; the weight and
+            // the free path do not change)
+            const JobDev& J = jobs[C.job[t]];
+            const BinDev& B = J.bins[C.bin[t]];
+            const double x64 = (1.0 - B.albedo_d) * B.kext_d * __ldg(J.rho64 + leaf) * Num<double>::pow2m(lev) *
+                               (double)tseg;
+            const double d64 = widen(W) * x64;
+            if (d64 > 0.0) {
+              if (dep_to) red_acc(dep_to + leaf, d64);
+              if (HITS && hitp) atomicAdd(hitp + leaf, 1u);
+              if (LEVELS && selfb && leaf == orig_t) atomicAdd(selfb + leaf, d64);
+            }
+          }
+        }
+      } else if (hit) {
+        tseg = tau / kev;
+      }
+      uint32_t moved;
+      const bool inside = cross_face(G, g, cur, leaf, E, tseg, !hit, dx, dy, dz, moved, P);
+      ev = hit ? EV_INTERACT : (inside ? EV_NONE : EV_ESCAPE);
+      if (!(E.t < Num<R>::inf())) ev = EV_DEGEN;  // cannot happen for |d| = 1
+      if (ev == EV_NONE) {
+        fetch_node();
+        if (MODE == 2 && (moved >> (lev + T.tsh)) != 0u) ev = EV_TILE;  // entered another tile: next round
+        // (the search for the neighbour starts at or above the level of the
+        // crossed face: cur.k <= that level)
+        if (LEVELS && cur.k < mlev) {
+          const int v = crossed_grid_level(g, E.x ? 0 : (E.y ? 1 : 2), dx, dy, dz);
+          if (v < mlev) {
+            const JobDev& J = jobs[C.job[t]];
+            if (v <= J.sub_conf) {
+              ev = EV_ESCAPE;  // left the subtree of this subiteration
+            } else {
+              mlev = v;
+              absb = J.absorbed ? J.absorbed + (long long)mlev * J.n_cells : nullptr;
+            }
+          }
+        }
+      }
+      if (EST == RT_EST_CONTINUOUS) {
+        R q, e;
+        Num<R>::absorb_given(x, ex, q, e);
+        const R dep = W * q;
+        W = W * e;
+        if (dep > R(0) && (sizeof(R) != 4 || kl >= R(FLT_MIN))) {
+          pkt_abs += dep;
+          if (dep_to) red_acc(dep_to + leaf, widen(dep));
+          if (HITS && hitp) atomicAdd(hitp + leaf, 1u);
+          if (LEVELS && selfb && leaf == orig_t) atomicAdd(selfb + leaf, widen(dep));
+        }
+      }
+      tau = hit ? R(0) : tau - tev;
+      ncross += tseg > R(0) ? 1u : 0u;
+    };
+    // every lane that leaves EV_NONE in the loop waits with an event
+    const int stay = max(0, __popc(__ballot_sync(FULL, ev == EV_NONE)) - (MODE == 2 ? RT_EV_BATCH_TILED : RT_EV_BATCH));
     if (RT_TRACE_ONLY_LOOP && (!PEEL || __ballot_sync(FULL, st == ST_PEEL) == 0u)) {
       do {
-        pass(std::true_type{});
-      } while (keep_stepping(ev, RT_EV_BATCH));
+        pass_trace();
+      } while (__popc(__ballot_sync(FULL, ev == EV_NONE)) > stay);
     } else {
       do {
-        pass(std::false_type{});
-      } while (keep_stepping(ev, RT_EV_BATCH));
+        pass();
+      } while (__popc(__ballot_sync(FULL, ev == EV_NONE)) > stay);
     }
 
     // ------------------------------------------------------------- slow path
@@ -1018,7 +1195,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
     const int job = C.job[t];
     if (ev == EV_KILL || (ev == EV_DEGEN && st == ST_TRACE)) {
       book_d(SL, jobs, job, wid, L_KILL, W);
-      book_u(SL, jobs, job, wid, U_KILL, 1ull);
+      book_u(SL, jobs, job, wid, U_KILL, 1u);
       atomicOr(&jobs[job].ledger->status, ev == EV_KILL ? 1 : 2);
       fate = 2;
     } else if (ev == EV_DEGEN || ev == EV_CUT) {
@@ -1107,7 +1284,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
         const R ua = draw(C, t);
         if (ua >= alb) {
           scatter = false;
-          if (absb) atomicAdd(absb + g.idx, widen(W));
+          if (absb) atomicAdd(absb + cur.pending, widen(W));
           pkt_abs += W;
           W = R(0);
           fate = 3;
@@ -1115,13 +1292,14 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
       }
       if (scatter) {
         C.nscat[t] += 1;
+        g.idx = cur.pending;
         bool inline_peel = PEEL && jobs[job].n_obs > 0;
         if (inline_peel && Q.cap > 0) {
           // defer: the peel-off kernel marches this record to every observer
           const unsigned long long slot = claim_slot(Q.count);
           if (slot < (unsigned long long)Q.cap) {
             PeelIO<R>::put(Q.rec, slot, g, dx, dy, dz, W, peel_meta(g.lev, C.bin[t], job));
-            book_u(SL, jobs, job, wid, U_DEFER, 1ull);
+            book_u(SL, jobs, job, wid, U_DEFER, 1u);
             inline_peel = false;
           }
         }
@@ -1151,6 +1329,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
       g.fx = C.sfx[t]; g.fy = C.sfy[t]; g.fz = C.sfz[t];
       cur.pending = g.idx;
       cur.k = g.lev;
+      fetch_node();
       P.n = 0;  // the stored path may be an inline peel-off march's
       const R sdx = C.sdx[t], sdy = C.sdy[t], sdz = C.sdz[t];
       int o = C.obs_i[t];
@@ -1161,7 +1340,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
         R pw;
         long long pix;
         if (!peel_setup<R>(J, o, g, sdx, sdy, sdz, W, C.gpar[t], C.bin[t], pw, pix)) {
-          book_u(SL, jobs, C.job[t], wid, U_POUT, 1ull);
+          book_u(SL, jobs, C.job[t], wid, U_POUT, 1u);
           continue;
         }
         C.pw[t] = pw;
@@ -1185,7 +1364,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
       const int job = C.job[t];
       book_d(SL, jobs, job, wid, L_ABS, pkt_abs);
       book_u(SL, jobs, job, wid, U_CROSS, ncross);
-      book_u(SL, jobs, job, wid, U_SCAT, (unsigned long long)C.nscat[t]);
+      book_u(SL, jobs, job, wid, U_SCAT, (uint32_t)C.nscat[t]);
       book_u(SL, jobs, job, wid, U_PCROSS, npeel);
       const long long li = C.log_index[t];
       if (li >= 0) {
@@ -1344,7 +1523,7 @@ __global__ void __launch_bounds__(256, PeelMinBlocks<R>::value) peel_kernel(cons
             }
             st = P_LIVE;
           } else {
-            book_u(SL, jobs, rjob, wid, U_POUT, 1ull);
+            book_u(SL, jobs, rjob, wid, U_POUT, 1u);
           }
         }
       }
@@ -1482,7 +1661,7 @@ __global__ void __launch_bounds__(256, PeelMinBlocks<R>::value) peel_kernel(cons
       book_d(SL, jobs, job, wid, L_PEEL, c);
     }
     if (ev == EV_ESCAPE || ev == EV_CUT) {
-      book_u(SL, jobs, job, wid, U_PCROSS, (unsigned long long)npeel);
+      book_u(SL, jobs, job, wid, U_PCROSS, npeel);
       st = P_DEAD;
     }
   }
