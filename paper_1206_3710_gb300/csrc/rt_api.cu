@@ -1080,11 +1080,25 @@ static int make_cfg(rt_ctx* c, int precision, bool peel, const rt_trace_params* 
   return RT_OK;
 }
 
-// Tiled tracing pays off when one wavelength's working set (4-byte node word
-// and 8-byte accumulator per cell) is well above the L2 (129 MB on GB300):
-// the root grid is cut into tiles of edge 2^tsh root cells whose working set
-// is at most 48 MB.  Single-job launches only.
-static bool choose_tiles(const rt_ctx* c, const rt_grid* G, int n_jobs, TileRun* T) {
+// Tiled tracing, single-job launches only.  Packages run bin by bin, so the
+// untiled tracer touches one wavelength's 4-byte node words and 8-byte
+// accumulators at a time; it stays near the rate of L2-resident cells while
+// the part of them in frequent use fits the L2 (129 MB on GB300).  A cell of
+// level l is crossed 4^-l times as often as a root cell (its cross-section),
+// so that part is counted as 12 B x sum n_l 4^-l.  Untiled against tiled
+// (20 wavelengths, one GB300): lognormal clouds of 31 MB (4.5e6 cells) 23.6
+// against 40.8 ms for 2e7 packages, of 112 MB (1.5e7 cells) 50.8 against 61.9
+// ms for 2e7 and 140 against 140 ms for 6e7, of 216 MB (2.4e7 cells) 28.1
+// against 33.2 ms for 4e6, 62.8 against 58.8 ms for 1e7 and 236 against 128 ms
+// for 4e7; the 9.2e6-cell disc (a few MB) 159 against 165 ms for 1e8.  With
+// few packages per bin every (bin, tile) pair of a round brings its cells
+// from DRAM for a handful of crossings: tiles need a package per bin for
+// every 48 counted cells.  The FP64 tracer is bound by the FP64 pipe either
+// way; it takes tiles where the whole grid exceeds one tile's 48 MB.
+// The tiles' edge: 2^tsh root cells, each tile's words and accumulators at
+// most 48 MB.
+static bool choose_tiles(const rt_ctx* c, const rt_grid* G, int n_jobs, int precision, int n_lambda, long long total,
+                         TileRun* T) {
   if (n_jobs != 1 || c->tile_edge == 0) return false;
   const int* R = G->root;
   auto count = [&](int edge) {
@@ -1092,8 +1106,11 @@ static bool choose_tiles(const rt_ctx* c, const rt_grid* G, int n_jobs, TileRun*
   };
   int edge = c->tile_edge;
   if (edge < 0) {
+    double n_use = 0.0;
+    for (int l = 0; l < G->n_levels; ++l) n_use += std::ldexp((double)(G->level_off[l + 1] - G->level_off[l]), -2 * l);
     const double ws = 12.0 * (double)G->n_cells, cap = 48.0 * 1024 * 1024;
     if (ws <= cap) return false;
+    if (precision == 32 && (12.0 * n_use <= 120.0e6 || 48.0 * ((double)total / n_lambda) < n_use)) return false;
     const double need = ws / cap;
     edge = 1;
     while (edge * 2 <= std::max(R[0], std::max(R[1], R[2]))) edge *= 2;
@@ -1254,7 +1271,7 @@ static int run_jobs(rt_ctx* c, int n_jobs, const TraceArgs* jobs, rt_ledger* led
     return fail(RT_ERR_INVALID, "hit counting needs rt_trace with the continuous estimator");
   const double to = launch_prm->timeout_s > 0 ? launch_prm->timeout_s : 3600.0;
   TileRun tiles;
-  bool tiled = !poly && total > 0 && n_items > 0 && choose_tiles(c, jobs[0].grid, n_jobs, &tiles);
+  bool tiled = !poly && total > 0 && n_items > 0 && choose_tiles(c, jobs[0].grid, n_jobs, precision, jobs[0].optics->n_lambda, total, &tiles);
   const bool split = n_jobs == 1 && jobs[0].prm->split_factor > 1;
   if (split && total > 0 && n_items > 0 && !tiled) {
     // resampling runs in the rounds of the tiled tracer: one tile

@@ -527,6 +527,34 @@ def test_tiled_equals_untiled(rt, case):
         assert led1[k] == pytest.approx(led0[k], rel=1e-12), k
 
 
+@pytest.mark.parametrize("root,npk,tiled", [
+    ((296, 224, 160), 300_000, True),   # 127 MB of root cells, more than a package for every 48 of them
+    ((296, 224, 160), 1_000, False),    # the same cells, too few packages
+    ((160, 160, 160), 300_000, False),  # 49 MB: the cells in use fit the L2
+])
+def test_automatic_tiles(rt, root, npk, tiled):
+    """The automatic choice between tiled and untiled tracing, and the same
+    field and counters from both."""
+    desc = synth.uniform_tree(root, tuple(float(n) for n in root), 1.0)
+    optics = synth.Optics(lambda_um=np.array([0.55]), kappa_ext=np.array([0.01]), albedo=np.array([0.5]),
+                          g_hg=np.array([0.3]), dnu=np.array([1e13]))
+    src = [synth.Source("external", bin_energy=np.array([1.0]))]
+    res = []
+    for edge in (-1, 0):
+        c = rt.Context(0)
+        c.set_tiles(edge)
+        g = rt.Grid(c, desc)
+        ab = _zeros(1, g.n_cells)
+        led = rt.rt_trace(c, g, src, optics, ab, seed=3, packets_per_bin=npk)
+        res.append((ab, led))
+    assert (res[0][1]["n_tiles"] > 0) == tiled and res[1][1]["n_tiles"] == 0
+    for k in ("n_packets", "n_cross", "n_scatter"):
+        assert res[0][1][k] == res[1][1][k], k
+    # FP64 sums of the same addends in another order: n eps of the largest cell
+    assert float((res[0][0] - res[1][0]).abs().max()) <= 1e-11 * float(res[1][0].max())
+
+
+
 @pytest.mark.parametrize("precision", [64, 32])
 def test_shards_are_one_run(rt, ctx, precision):
     """Launches with package offsets 0 and n are, package by package, the two
