@@ -80,7 +80,8 @@ struct rt_ctx {
   DevBuf table;        // job tables
   DevBuf small;        // ledgers + counter
   DevBuf scan_tmp;
-  DevBuf dust_arrays;  // lambda, kappa_abs, dnu, temperature table
+  DevBuf dust_arrays;  // lambda, kappa_abs, dnu of a dust source
+  DevBuf dust_tab;     // lambda, kappa_abs, dnu and the temperature tables
   DevBuf lam;          // Lambda iteration: stored fields, previous T, hits
   std::vector<DevBuf> cdf;  // per dust source
   void* pinned = nullptr;
@@ -198,6 +199,7 @@ extern "C" void rt_ctx_destroy(rt_ctx* c) {
   c->small.release();
   c->scan_tmp.release();
   c->dust_arrays.release();
+  c->dust_tab.release();
   c->lam.release();
   for (auto& b : c->cdf) b.release();
   if (c->pinned) cudaFreeHost(c->pinned);
@@ -574,25 +576,27 @@ static const rt_dust* resolve_dust(const rt_dust* du, const rt_optics* op, std::
   return &out;
 }
 
-// upload lambda, kappa_abs, dnu into ctx->dust_arrays (+ table of n_table)
-static int upload_dust(rt_ctx* c, const rt_dust* du, int n_table, double** lam, double** kab, double** dnu,
+// upload lambda, kappa_abs, dnu into buf, with room for the tables of n_table
+// nodes behind them
+static int upload_dust(rt_ctx* c, DevBuf& buf, const rt_dust* du, int n_table, double** lam, double** kab, double** dnu,
                        double** table, cudaStream_t s) {
   const int nl = du->n_lambda;
-  const size_t bytes = sizeof(double) * (3 * (size_t)nl + 3 * (size_t)n_table) + 256;
-  int rc = c->dust_arrays.ensure(bytes);
+  const size_t n_tab = n_table > 0 ? dust_table_doubles(n_table) + 8 : 0;
+  const size_t bytes = sizeof(double) * (3 * (size_t)nl + n_tab) + 256;
+  int rc = buf.ensure(bytes);
   if (rc) return rc;
-  rc = ensure_pinned(c, bytes);
+  rc = ensure_pinned(c, sizeof(double) * 3 * (size_t)nl);
   if (rc) return rc;
   double* hp = reinterpret_cast<double*>(c->pinned);
   memcpy(hp, du->lambda_um, sizeof(double) * nl);
   memcpy(hp + nl, du->kappa_abs, sizeof(double) * nl);
   memcpy(hp + 2 * nl, du->dnu, sizeof(double) * nl);
-  double* dp = reinterpret_cast<double*>(c->dust_arrays.p);
+  double* dp = reinterpret_cast<double*>(buf.p);
   CK(cudaMemcpyAsync(dp, hp, sizeof(double) * 3 * nl, cudaMemcpyHostToDevice, s));
   *lam = dp;
   *kab = dp + nl;
   *dnu = dp + 2 * nl;
-  *table = dp + 3 * nl;
+  *table = dp + (3 * (size_t)nl + 7) / 8 * 8;  // 64-byte aligned
   return RT_OK;
 }
 
@@ -744,11 +748,11 @@ static int build_tables(rt_ctx* c, int n_jobs, const TraceArgs* jobs, LedgerDev*
         rc = cb.ensure(sizeof(double) * ((size_t)nl * nc + (size_t)nl * (nc + 1) + 2 * (size_t)nl) + 256);
         if (rc) return rc;
         double *lam, *kab, *dnu, *tab;
-        rc = upload_dust(c, S.dust, 0, &lam, &kab, &dnu, &tab, s);
+        rc = upload_dust(c, c->dust_arrays, S.dust, 0, &lam, &kab, &dnu, &tab, s);
         if (rc) return rc;
         double* em = reinterpret_cast<double*>(cb.p);
         double* tot = em + (size_t)nl * nc + (size_t)nl * (nc + 1);
-        CK(dust_emission(S.T_dev, nc, G->child, G->rho64, G->level, G->h0, lam, kab, dnu, nl, em, s));
+        CK(dust_emission(S.T_dev, nc, G->child, G->rho64, G->level, G->h0, lam, kab, dnu, nl, em, c->sm_count, s));
         CK(row_sums_f64(em, nl, nc, tot, s));
         rc = ensure_pin_rb(c, sizeof(double) * (size_t)nl);
         if (rc) return rc;
@@ -824,11 +828,10 @@ static int build_tables(rt_ctx* c, int n_jobs, const TraceArgs* jobs, LedgerDev*
       if (rc) return rc;
       memcpy(c->pinned, w_dust.data() + (size_t)si * nl, sizeof(double) * (size_t)nl);
       CK(cudaMemcpyAsync(wd, c->pinned, sizeof(double) * (size_t)nl, cudaMemcpyHostToDevice, s));
-      CK(dust_counts(em, nc, nl, wd, (uint32_t)p->seed ^ p->job, (uint32_t)(p->seed >> 32) ^ p->iter, (uint32_t)si,
-                     first, s));
-      rc = c->scan_tmp.ensure(scan_rows_tmp_bytes(nl, nc + 1));
+      rc = c->scan_tmp.ensure(dust_counts_tmp_bytes(nl, nc));
       if (rc) return rc;
-      CK(scan_rows_i64_excl(first, nl, nc + 1, c->scan_tmp.p, c->scan_tmp.n, s));
+      CK(dust_counts(em, nc, nl, wd, (uint32_t)p->seed ^ p->job, (uint32_t)(p->seed >> 32) ^ p->iter, (uint32_t)si,
+                     first, c->scan_tmp.p, c->scan_tmp.n, s));
       rc = ensure_pin_rb(c, sizeof(long long) * (size_t)nl);
       if (rc) return rc;
       for (int b = 0; b < nl; ++b)
@@ -1514,11 +1517,11 @@ extern "C" int rt_dust_temperature(rt_ctx* ctx, const rt_grid* g, const double* 
   cudaStream_t s = (cudaStream_t)cuda_stream;
   const int n_table = 8192;
   double *lam, *kab, *dnu, *tab;
-  rc = upload_dust(ctx, dust, n_table, &lam, &kab, &dnu, &tab, s);
+  rc = upload_dust(ctx, ctx->dust_tab, dust, n_table, &lam, &kab, &dnu, &tab, s);
   if (rc) return rc;
   CK(dust_table(lam, kab, dnu, dust->n_lambda, dust->T_min, dust->T_max, n_table, tab, s));
   CK(dust_temperature(absorbed_dev, n_bins, g->n_cells, g->child, g->rho64, g->level, g->h0, lam, kab, dnu,
-                      dust->n_lambda, dust->T_min, dust->T_max, tab, n_table, T_dev, s));
+                      dust->n_lambda, dust->T_min, dust->T_max, tab, n_table, T_dev, ctx->sm_count, s));
   CK(cudaEventRecord(ctx->ev_b, s));
   return ctx_wait(ctx, ctx->ev_b, 3600.0);
 }
@@ -1533,9 +1536,10 @@ extern "C" int rt_dust_emission(rt_ctx* ctx, const rt_grid* g, const double* T_d
   DeviceGuard dg(ctx->device);
   cudaStream_t s = (cudaStream_t)cuda_stream;
   double *lam, *kab, *dnu, *tab;
-  rc = upload_dust(ctx, dust, 0, &lam, &kab, &dnu, &tab, s);
+  rc = upload_dust(ctx, ctx->dust_arrays, dust, 0, &lam, &kab, &dnu, &tab, s);
   if (rc) return rc;
-  CK(dust_emission(T_dev, g->n_cells, g->child, g->rho64, g->level, g->h0, lam, kab, dnu, dust->n_lambda, emission_dev, s));
+  CK(dust_emission(T_dev, g->n_cells, g->child, g->rho64, g->level, g->h0, lam, kab, dnu, dust->n_lambda,
+                   emission_dev, ctx->sm_count, s));
   const size_t tb = sizeof(double) * (size_t)dust->n_lambda;
   if (bin_total_host) {
     rc = ctx->small.ensure(tb + 256);
@@ -1682,13 +1686,16 @@ extern "C" int rt_lambda_iterate(rt_ctx* ctx, const rt_grid* g, int n_src, const
   if (rc && rc != RT_ERR_STEP_LIMIT) return rc;
 
   const int n_table = 8192;
+  // the dust model's tables, made at the first solve
+  double *lam = nullptr, *kab, *dnu, *tab;
   auto solve = [&](const double* absorbed) -> int {
-    double *lam, *kab, *dnu, *tab;
-    int r = upload_dust(ctx, du, n_table, &lam, &kab, &dnu, &tab, s);
-    if (r) return r;
-    CK(dust_table(lam, kab, dnu, du->n_lambda, du->T_min, du->T_max, n_table, tab, s));
+    if (!lam) {
+      int r = upload_dust(ctx, ctx->dust_tab, du, n_table, &lam, &kab, &dnu, &tab, s);
+      if (r) return r;
+      CK(dust_table(lam, kab, dnu, du->n_lambda, du->T_min, du->T_max, n_table, tab, s));
+    }
     CK(dust_temperature(absorbed, 1, nc, g->child, g->rho64, g->level, g->h0, lam, kab, dnu, du->n_lambda, du->T_min,
-                        du->T_max, tab, n_table, T_dev, s));
+                        du->T_max, tab, n_table, T_dev, ctx->sm_count, s));
     return RT_OK;
   };
   rc = solve(A_star);
@@ -1804,18 +1811,16 @@ extern "C" int rt_lambda_subiterate(rt_ctx* ctx, const rt_grid* g, int n_src, co
   CK(cudaMemcpyAsync(A, A_star, fb, cudaMemcpyDeviceToDevice, s));
 
   const int n_table = 8192;
-  double *lam, *kab, *dnu, *tab;
-  auto upload = [&]() -> int {
-    int r = upload_dust(ctx, du, n_table, &lam, &kab, &dnu, &tab, s);
-    if (r) return r;
-    CK(dust_table(lam, kab, dnu, du->n_lambda, du->T_min, du->T_max, n_table, tab, s));
-    return RT_OK;
-  };
+  // the dust model's tables, made at the first solve
+  double *lam = nullptr, *kab, *dnu, *tab;
   auto solve = [&](const double* absorbed) -> int {
-    int r = upload();
-    if (r) return r;
+    if (!lam) {
+      int r = upload_dust(ctx, ctx->dust_tab, du, n_table, &lam, &kab, &dnu, &tab, s);
+      if (r) return r;
+      CK(dust_table(lam, kab, dnu, du->n_lambda, du->T_min, du->T_max, n_table, tab, s));
+    }
     CK(dust_temperature(absorbed, 1, nc, g->child, g->rho64, g->level, g->h0, lam, kab, dnu, du->n_lambda, du->T_min,
-                        du->T_max, tab, n_table, T_dev, s));
+                        du->T_max, tab, n_table, T_dev, ctx->sm_count, s));
     return RT_OK;
   };
   auto read_scalars = [&](double* out, int n) -> int {
@@ -1850,8 +1855,6 @@ extern "C" int rt_lambda_subiterate(rt_ctx* ctx, const rt_grid* g, int n_src, co
     // emission at levels <= L and below L with the current temperatures
     double e[7] = {0, 0, 0, 0, 0, 0, 0};
     if (it > 1) {
-      rc = upload();
-      if (rc) return rc;
       CK(level_imbalance(A, T_dev, g->child, g->rho64, g->level, g->h0, tab, n_table, nc, L, scal + 1, s));
       rc = read_scalars(e, 7);
       if (rc) return rc;
@@ -1882,9 +1885,8 @@ extern "C" int rt_lambda_subiterate(rt_ctx* ctx, const rt_grid* g, int n_src, co
     // send in a full step
     std::vector<double> w_full;
     if (kind == 1) {
-      rc = upload();
-      if (rc) return rc;
-      CK(dust_emission_totals(T_dev, nc, g->child, g->rho64, g->level, g->h0, lam, kab, dnu, nlb, scal + 16, s));
+      CK(dust_emission_totals(T_dev, nc, g->child, g->rho64, g->level, g->h0, lam, kab, dnu, nlb, scal + 16,
+                              ctx->sm_count, s));
       rc = ensure_pin_rb(ctx, sizeof(double) * (size_t)nlb);
       if (rc) return rc;
       CK(cudaMemcpyAsync(ctx->pin_rb, scal + 16, sizeof(double) * (size_t)nlb, cudaMemcpyDeviceToHost, s));
@@ -1921,8 +1923,6 @@ extern "C" int rt_lambda_subiterate(rt_ctx* ctx, const rt_grid* g, int n_src, co
                        cudaMemcpyDeviceToDevice, s));
     CK(sum_levels(I, nlev, nc, A_star, A, s));
     // imbalance of the new field against the emission that produced it
-    rc = upload();
-    if (rc) return rc;
     CK(level_imbalance(A, T_prev, g->child, g->rho64, g->level, g->h0, tab, n_table, nc, L, scal + 1, s));
     rc = solve(A);
     if (!rc && sp->ali) {
@@ -1932,7 +1932,7 @@ extern "C" int rt_lambda_subiterate(rt_ctx* ctx, const rt_grid* g, int n_src, co
       CK(ali_weights(A, self_abs, self_emit, self_cnt, kab, (unsigned)std::max(1, sp->ali_min_packages), lam_max,
                      nlb, nc, ali_rhs, ali_w, ali_use, s));
       CK(dust_temperature_weighted(ali_rhs, ali_w, ali_use, nc, g->child, g->rho64, g->level, g->h0, lam, kab, dnu,
-                                   du->n_lambda, du->T_min, du->T_max, T_dev, s));
+                                   du->n_lambda, du->T_min, du->T_max, T_dev, ctx->sm_count, s));
     }
     if (rc) return rc;
     CK(max_rel_change(T_dev, T_prev, hits_step, g->child, nc, lp->min_hits, scal, s));

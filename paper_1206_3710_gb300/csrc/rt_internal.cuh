@@ -319,14 +319,16 @@ cudaError_t dust_table(const double* lam_um, const double* kabs, const double* d
 cudaError_t dust_temperature(const double* absorbed, int n_bins, long long n_cells, const uint32_t* child,
                              const double* rho64, const uint8_t* level, double h0, const double* lam_um,
                              const double* kabs, const double* dnu, int nl, double Tmin, double Tmax,
-                             const double* table, int n_table, double* T, cudaStream_t s);
+                             const double* table, int n_table, double* T, int sm_count, cudaStream_t s);
+// doubles that dust_table's tables take for n_table nodes
+size_t dust_table_doubles(int n_table);
 cudaError_t dust_emission(const double* T, long long n_cells, const uint32_t* child, const double* rho64,
                           const uint8_t* level, double h0, const double* lam_um, const double* kabs,
-                          const double* dnu, int nl, double* emission, cudaStream_t s);
+                          const double* dnu, int nl, double* emission, int sm_count, cudaStream_t s);
 // per-bin totals of dust_emission's emission into tot [nl] (device)
 cudaError_t dust_emission_totals(const double* T, long long n_cells, const uint32_t* child, const double* rho64,
                                  const uint8_t* level, double h0, const double* lam, const double* kabs,
-                                 const double* dnu, int nl, double* tot, cudaStream_t s);
+                                 const double* dnu, int nl, double* tot, int sm_count, cudaStream_t s);
 // max over leaves with hits >= min_hits of |T - T_prev| / T_prev into *out
 cudaError_t max_rel_change(const double* T, const double* T_prev, const unsigned int* hits, const uint32_t* child,
                            long long n, double min_hits, double* out, cudaStream_t s);
@@ -346,7 +348,7 @@ cudaError_t ali_weights(const double* A, const double* self, const double* emitt
 cudaError_t dust_temperature_weighted(const double* rhs, const double* w, const uint8_t* use, long long n,
                                       const uint32_t* child, const double* rho64, const uint8_t* level, double h0,
                                       const double* lam, const double* kabs, const double* dnu, int nl, double Tmin,
-                                      double Tmax, double* T, cudaStream_t s);
+                                      double Tmax, double* T, int sm_count, cudaStream_t s);
 cudaError_t level_imbalance(const double* A, const double* T, const uint32_t* child, const double* rho64,
                             const uint8_t* level, double h0, const double* table, int n_table, long long n, int L,
                             double* out, cudaStream_t s);
@@ -359,12 +361,13 @@ size_t scan_rows_tmp_bytes(int n_rows, long long n);
 // exclusive prefix sums of n_rows rows of length n (int64), in place
 cudaError_t scan_rows_i64_excl(long long* data, int n_rows, long long n, void* tmp, size_t tmp_bytes,
                                cudaStream_t s);
-// Dust packages per cell (Sect. 4.2): row b of first [nl][n + 1] gets, for
-// each cell, floor(emission[b][c] / w[b] + u_bc) (u_bc: word 0 of Philox
-// counter (c, 0x80000000, 0, (src << 16) | b) under key (k0, k1)), and 0 in
-// the last column; an exclusive scan of the rows then gives each cell's
-// first package and the bin's total.  w: device [nl]; w[b] <= 0: no packages
+// Dust packages per cell (Sect. 4.2): cell c sends floor(emission[b][c] /
+// w[b] + u_bc) packages of bin b (u_bc: word 0 of Philox counter (c,
+// 0x80000000, 0, (src << 16) | b) under key (k0, k1)); row b of first
+// [nl][n + 1] gets each cell's first package and, in the last column, the
+// bin's total.  w: device [nl]; w[b] <= 0: no packages
 cudaError_t dust_counts(const double* emission, long long n, int nl, const double* w, uint32_t k0, uint32_t k1,
-                        uint32_t src, long long* first, cudaStream_t s);
+                        uint32_t src, long long* first, void* tmp, size_t tmp_bytes, cudaStream_t s);
+size_t dust_counts_tmp_bytes(int nl, long long n);
 
 }  // namespace rtk

@@ -712,6 +712,63 @@ def test_dust_temperature_parity_ranges(rt, ctx, orc, n_lambda, T_min, T_max):
     np.testing.assert_allclose(To[inside], T_true[inside], rtol=1e-9)
 
 
+@pytest.mark.parametrize("n", [1, 255, 1023, 1024, 1025, 2049])
+def test_dust_packages_at_chunk_edges(rt, ctx, orc, n):
+    """Packages per cell, floor(E / w + u), at the edges of the chunks the
+    counts are taken in: the launch sends their sum, and each package starts
+    in the cell that the exclusive sums give it."""
+    desc = synth.uniform_tree((n, 1, 1), (n * 1e15, 1e15, 1e15), 1e-19)
+    g = rt.Grid(ctx, desc)
+    lam = np.array([3.0, 30.0, 300.0])
+    kabs, dnu = np.array([100.0, 10.0, 0.1]), synth.bin_dnu(lam)
+    T = np.random.default_rng(n).uniform(0.0, 60.0, n)
+    Td = torch.from_numpy(T).to(DEV)
+    em = _zeros(3, n)
+    tot = rt.rt_dust_emission(ctx, g, Td, lam, kabs, dnu, em)
+    em = em.cpu().numpy()
+    budget, seed = 5 * n + 7, 17
+    u = np.array([[orc.philox4x32(np.array([c, 0x80000000, 0, b], np.uint32), np.array([seed, 0], np.uint32))[0]
+                   for c in range(n)] for b in range(3)], dtype=np.float64)
+    k = np.floor(em / (tot / budget)[:, None] + (u + 0.5) * 2.0 ** -32).astype(np.int64)
+    # an opaque, purely absorbing medium: a package stays in its own cell, so
+    # the hits are the packages of each cell
+    optics = synth.Optics(lambda_um=lam, kappa_ext=np.full(3, 1e12), albedo=np.zeros(3), g_hg=np.zeros(3), dnu=dnu)
+    log = _zeros(3 * budget + 3 * n, 10)
+    led = rt.rt_trace(ctx, g, [rt.DustSource(Td, lam, kabs, dnu)], optics, _zeros(3, n), seed=seed, precision=64,
+                      packets_per_bin=budget, packet_log=log)
+    assert led["n_packets"] == k.sum()
+    lg = log.cpu().numpy()[:led["n_packets"]]
+    # every package was traced (an unset row has no direction)
+    assert np.allclose((lg[:, 7:] ** 2).sum(axis=1), 1.0)
+
+
+@pytest.mark.parametrize("x", [1e-6, 1 / 371.0, 1 / 369.0, 0.05, 1.0, 44.0, 45.0, 700.0, 706.9, 707.1, 709.7, 709.8, 3000.0])
+def test_dust_emission_edges(rt, ctx, orc, x):
+    """Emission where the integer form of the Planck term begins and ends
+    (x = h nu / kT near 1/370, 707 and 709.78) and between, against the
+    oracle's FP64 sum.  Both round x to a few eps (8 taken), which moves the
+    term by x times that; subnormal factors above 707 by far more."""
+    desc = synth.random_refined_tree((4, 3, 5), (4e16, 3e16, 5e16), 2, 0.3, 3,
+                                     rho_fn=lambda l, a, b, c: 10.0 ** np.random.default_rng(l).uniform(-24, -18, a.size))
+    g = rt.Grid(ctx, desc)
+    tree = orc.Tree(desc)
+    lam = np.array([0.5, 20.0])
+    kabs, dnu = np.array([50.0, 3.0]), synth.bin_dnu(lam)
+    hck = synth.H_CGS * synth.C_CGS / synth.K_CGS / 1e-4   # um K
+    spread = np.random.default_rng(1).uniform(0.9999, 1.0001, desc.n_cells)
+    T = hck / (lam[0] * x) * spread
+    T[:3] = [0.0, 1e-3, 2.7]
+    em = _zeros(2, desc.n_cells)
+    tot = rt.rt_dust_emission(ctx, g, torch.from_numpy(T).to(DEV), lam, kabs, dnu, em)
+    eo = orc.dust_emission(tree, T, lam, kabs, dnu)
+    eg = em.cpu().numpy()
+    for b in range(2):
+        xb = x * lam[0] / lam[b]
+        tol = 8 * 2.2e-16 * (1.0 + 1.001 * xb) if xb < 706.0 else 1e-3
+        np.testing.assert_allclose(eg[b][3:], eo[b][3:], rtol=tol, atol=1e-290 if xb > 706.0 else 0.0)
+    np.testing.assert_allclose(tot, eg.sum(axis=1), rtol=1e-13)
+
+
 def test_fp64_dust_source_per_packet(rt, ctx, orc):
     L = 20 * synth.AU_CM
     desc = synth.random_refined_tree((6, 6, 6), (L,) * 3, 2, 0.3, 4,
