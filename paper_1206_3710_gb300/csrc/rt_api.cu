@@ -753,7 +753,7 @@ static int build_tables(rt_ctx* c, int n_jobs, const TraceArgs* jobs, LedgerDev*
         double* em = reinterpret_cast<double*>(cb.p);
         double* tot = em + (size_t)nl * nc + (size_t)nl * (nc + 1);
         CK(dust_emission(S.T_dev, nc, G->child, G->rho64, G->level, G->h0, lam, kab, dnu, nl, em, c->sm_count, s));
-        CK(row_sums_f64(em, nl, nc, tot, s));
+        CK(row_sums_f64(em, nl, nc, tot, c->sm_count, s));
         rc = ensure_pin_rb(c, sizeof(double) * (size_t)nl);
         if (rc) return rc;
         CK(cudaMemcpyAsync(c->pin_rb, tot, sizeof(double) * (size_t)nl, cudaMemcpyDeviceToHost, s));
@@ -1546,7 +1546,7 @@ extern "C" int rt_dust_emission(rt_ctx* ctx, const rt_grid* g, const double* T_d
     if (!rc) rc = ensure_pin_rb(ctx, tb);
     if (rc) return rc;
     double* tot = reinterpret_cast<double*>(ctx->small.p);
-    CK(row_sums_f64(emission_dev, dust->n_lambda, g->n_cells, tot, s));
+    CK(row_sums_f64(emission_dev, dust->n_lambda, g->n_cells, tot, ctx->sm_count, s));
     CK(cudaMemcpyAsync(ctx->pin_rb, tot, tb, cudaMemcpyDeviceToHost, s));
   }
   CK(cudaEventRecord(ctx->ev_b, s));

@@ -530,6 +530,34 @@ __device__ __forceinline__ void red_acc(double* p, double v) {
 #endif
 }
 
+// The same for lanes that are likely to meet in one cell: the lanes that call
+// together and share an address are summed in registers (a tree over each
+// group), and one of them updates the accumulator, and the hit counter with
+// the number of lanes.  The L2 takes reductions to one address one after
+// another, 1.5 ns each, and every access queued behind them waits; the first
+// cells around a point source or under a beam take all its packages.  Not
+// for every deposit: finding the groups costs some 80 cycles of the SM.
+__device__ __forceinline__ void red_acc_grouped(double* p, unsigned int* hits, double v) {
+  const unsigned m = __activemask();
+  const int lane = threadIdx.x & 31;
+  unsigned peers = __match_any_sync(m, (unsigned long long)(p ? (uintptr_t)p : (uintptr_t)hits));
+  const unsigned n = (unsigned)__popc(peers);
+  const bool lead = lane == __ffs(peers) - 1;
+  unsigned rank = (unsigned)__popc(peers & ((1u << lane) - 1u));
+  peers &= ~((2u << lane) - 1u);  // the group's lanes after this one
+  while (__any_sync(m, peers != 0u)) {
+    const int next = __ffs(peers);
+    const double t = __shfl_sync(m, v, next ? next - 1 : lane);
+    if (next) v += t;
+    peers &= __ballot_sync(m, (rank & 1u) == 0u);
+    rank >>= 1;
+  }
+  if (lead) {
+    if (p) red_acc(p, v);
+    if (hits) atomicAdd(hits, n);
+  }
+}
+
 // f32 -> f64 for the accumulator reductions (one conversion per deposit;
 // measured as fast as assembling the f64 bits on the integer pipe)
 __device__ __forceinline__ double widen(float v) { return (double)v; }

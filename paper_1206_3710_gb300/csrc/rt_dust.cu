@@ -461,7 +461,7 @@ cudaError_t max_rel_change(const double* T, const double* T_prev, const unsigned
                            long long n, double min_hits, double* out, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(out, 0, sizeof(double), s);
   if (e != cudaSuccess) return e;
-  max_rel_change_kernel<<<1024, 256, 0, s>>>(T, T_prev, hits, child, n, min_hits, out);
+  max_rel_change_kernel<<<(unsigned)std::min<long long>((n + 255) / 256, 1024), 256, 0, s>>>(T, T_prev, hits, child, n, min_hits, out);
   return cudaGetLastError();
 }
 
@@ -576,22 +576,38 @@ cudaError_t dust_counts(const double* emission, long long n, int nl, const doubl
   return cudaGetLastError();
 }
 
-__global__ void row_sum_kernel(const double* __restrict__ data, long long n, double* __restrict__ out) {
+// One atomic per block: with one per warp and 512 blocks a row, the 1.2e5
+// atomics to 30 addresses of a 30-bin row set took 145 us whatever the rows'
+// length.
+__global__ void __launch_bounds__(256) row_sum_kernel(const double* __restrict__ data, long long n,
+                                                      double* __restrict__ out) {
+  __shared__ double part[8];
   const long long row = blockIdx.y;
-  double v = 0.0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    v += data[row * n + i];
+  const double* d = data + row * n;
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  double v = 0.0, v2 = 0.0;
+  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  for (; i + stride < n; i += 2 * stride) {
+    v += d[i];
+    v2 += d[i + stride];
+  }
+  if (i < n) v += d[i];
+  v += v2;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-  if ((threadIdx.x & 31) == 0 && v != 0.0) atomicAdd(out + row, v);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < 8; ++k) v += part[k];
+    if (v != 0.0) atomicAdd(out + row, v);
+  }
 }
 
-cudaError_t row_sums_f64(const double* data, int n_rows, long long n, double* out, cudaStream_t s) {
+cudaError_t row_sums_f64(const double* data, int n_rows, long long n, double* out, int sm_count, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(out, 0, sizeof(double) * (size_t)n_rows, s);
   if (e != cudaSuccess) return e;
-  long long blocks = (n + 255) / 256;
-  if (blocks > 512) blocks = 512;
-  if (blocks < 1) blocks = 1;
+  // at least 16 values a thread, and eight blocks per SM over the rows
+  const long long blocks = std::max<long long>(1, std::min<long long>((n + 4095) / 4096, (8ll * sm_count + n_rows - 1) / n_rows));
   row_sum_kernel<<<dim3((unsigned)blocks, n_rows), 256, 0, s>>>(data, n, out);
   return cudaGetLastError();
 }
@@ -808,11 +824,18 @@ __global__ void imbalance_kernel(const double* __restrict__ A, const double* __r
     v[gi + 1] += mass;
     v[4 + gi / 2] += mass * E;
   }
+  __shared__ double part[6][8];
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
     double x = v[k];
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
-    if ((threadIdx.x & 31) == 0 && x != 0.0) atomicAdd(out + k, x);
+    if ((threadIdx.x & 31) == 0) part[k][threadIdx.x >> 5] = x;
+  }
+  __syncthreads();
+  if (threadIdx.x < 6) {
+    double x = 0.0;
+    for (int k = 0; k < 8; ++k) x += part[threadIdx.x][k];
+    if (x != 0.0) atomicAdd(out + threadIdx.x, x);
   }
 }
 
@@ -821,7 +844,7 @@ cudaError_t level_imbalance(const double* A, const double* T, const uint32_t* ch
                             double* out, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(out, 0, 6 * sizeof(double), s);
   if (e != cudaSuccess) return e;
-  imbalance_kernel<<<1024, 256, 0, s>>>(A, T, child, rho64, level, h0, table, n_table, n, L, out);
+  imbalance_kernel<<<(unsigned)std::min<long long>((n + 255) / 256, 1024), 256, 0, s>>>(A, T, child, rho64, level, h0, table, n_table, n, L, out);
   return cudaGetLastError();
 }
 

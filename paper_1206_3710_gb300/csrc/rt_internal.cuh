@@ -353,7 +353,7 @@ cudaError_t level_imbalance(const double* A, const double* T, const uint32_t* ch
                             const uint8_t* level, double h0, const double* table, int n_table, long long n, int L,
                             double* out, cudaStream_t s);
 // per-row sums of rows x n (f64) into out[rows] (device)
-cudaError_t row_sums_f64(const double* data, int n_rows, long long n, double* out, cudaStream_t s);
+cudaError_t row_sums_f64(const double* data, int n_rows, long long n, double* out, int sm_count, cudaStream_t s);
 // inclusive prefix sums of n_rows rows of length n (f64), in place
 cudaError_t scan_rows_f64(double* data, int n_rows, long long n, void* tmp, size_t tmp_bytes,
                           cudaStream_t s);
