@@ -1154,7 +1154,7 @@ static int run_tiled(rt_ctx* c, TileRun T, int n_lambda, int precision, bool pee
   int rc = c->tile_a.ensure(rb * (size_t)rec_cap);
   if (!rc) rc = c->tile_b.ensure(rb * (size_t)rec_cap);
   if (!rc) rc = c->tile_key.ensure(sizeof(uint32_t) * (size_t)rec_cap);
-  if (!rc) rc = c->tile_hist.ensure(sizeof(unsigned long long) * ((size_t)n_keys + 1));
+  if (!rc) rc = c->tile_hist.ensure(tile_hist_bytes(n_keys));
   if (rc) return rc;
   T.out_key = reinterpret_cast<uint32_t*>(c->tile_key.p);
   T.n_out = n_out;
@@ -1203,23 +1203,34 @@ static int run_tiled(rt_ctx* c, TileRun T, int n_lambda, int precision, bool pee
 // Deferred peel-off records sorted by block of root cells (at most
 // RT_PEEL_SORT_KEYS blocks of the first job's root grid: 4^3 root cells on a
 // 256^3 root), so that the lanes of a warp march from nearby points: the
-// queue length is read back (the tracer has finished), the records are
-// counting-sorted into a second buffer.
+// records are counting-sorted into a second buffer.  A queue of at most
+// RT_PEEL_SORT_BLIND records gets a second buffer of its whole capacity and
+// its length stays on the device: reading it back would leave the GPU idle
+// for the wait and the launches behind it.  For a longer queue that wait is
+// small beside the march, and the buffer takes only the records there are.
 #ifndef RT_PEEL_SORT
 #define RT_PEEL_SORT 1
 #endif
 #ifndef RT_PEEL_SORT_KEYS
 #define RT_PEEL_SORT_KEYS 262144
 #endif
+#ifndef RT_PEEL_SORT_BLIND
+#define RT_PEEL_SORT_BLIND (1ll << 22)
+#endif
 static int sort_peel_queue(rt_ctx* c, const PeelQueue& q, int precision, const rt_grid* G, double timeout_s,
                            cudaStream_t s, PeelQueue* out, long long* launches) {
   *out = q;
-  CK(cudaMemcpyAsync(c->pin_count, q.count, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-  CK(cudaEventRecord(c->ev_c, s));
-  int rc = ctx_wait(c, c->ev_c, timeout_s);
-  if (rc) return rc;
-  const long long n = std::min<long long>((long long)c->pin_count[0], q.cap);
-  if (n < 64) return RT_OK;
+  const bool blind = q.cap <= RT_PEEL_SORT_BLIND;
+  long long n = q.cap;
+  int rc = RT_OK;
+  if (!blind) {
+    CK(cudaMemcpyAsync(c->pin_count, q.count, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+    CK(cudaEventRecord(c->ev_c, s));
+    rc = ctx_wait(c, c->ev_c, timeout_s);
+    if (rc) return rc;
+    n = std::min<long long>((long long)c->pin_count[0], q.cap);
+    if (n < 64) return RT_OK;
+  }
   int bs = 0;
   auto nb = [&](int r) { return (r + (1 << bs) - 1) >> bs; };
   while ((long long)nb(G->root[0]) * nb(G->root[1]) * nb(G->root[2]) > RT_PEEL_SORT_KEYS) ++bs;
@@ -1227,18 +1238,17 @@ static int sort_peel_queue(rt_ctx* c, const PeelQueue& q, int precision, const r
   const size_t rb = peel_record_bytes(precision);
   rc = c->peel_q2.ensure(rb * (size_t)n);
   if (!rc) rc = c->tile_key.ensure(sizeof(uint32_t) * (size_t)n);
-  if (!rc) rc = c->tile_hist.ensure(sizeof(unsigned long long) * ((size_t)n_keys + 1));
+  if (!rc) rc = c->tile_hist.ensure(tile_hist_bytes(n_keys));
   if (rc == RT_ERR_OOM) {
     cudaGetLastError();  // no room for the sorted copy: march the queue as it is
     return RT_OK;
   }
   if (rc) return rc;
-  uint32_t* key = reinterpret_cast<uint32_t*>(c->tile_key.p);
-  CK(peel_keys(precision, q.rec, n, bs, nb(G->root[0]), nb(G->root[1]), nb(G->root[2]), key, c->sm_count, s));
-  CK(tile_sort(q.rec, key, n, (int)rb, n_keys, reinterpret_cast<unsigned long long*>(c->tile_hist.p), c->peel_q2.p,
-               s));
+  CK(peel_sort(precision, q.rec, n, blind ? q.count : nullptr, bs, nb(G->root[0]), nb(G->root[1]), nb(G->root[2]),
+               reinterpret_cast<uint32_t*>(c->tile_key.p), reinterpret_cast<unsigned long long*>(c->tile_hist.p),
+               c->peel_q2.p, c->sm_count, s));
   out->rec = c->peel_q2.p;
-  *launches += 4;  // keys, histogram, scan, scatter
+  *launches += 3;  // keys and histogram, scan, scatter
   return RT_OK;
 }
 

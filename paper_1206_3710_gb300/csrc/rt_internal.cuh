@@ -247,7 +247,8 @@ size_t tile_record_bytes(int precision, bool wide);
 cudaError_t launch_poly(int precision, int group, bool peel, const JobDev* jobs, const ItemDev* items, int n_items,
                         unsigned long long* counter, long long total, int sm_count, cudaStream_t s);
 // counting sort of n records (rec_bytes each) by key (< n_keys) from in/key
-// into out; hist_dev holds n_keys + 1 counters
+// into out; hist_dev: tile_hist_bytes(n_keys)
+size_t tile_hist_bytes(int n_keys);
 cudaError_t tile_sort(const void* in, const uint32_t* key, long long n, int rec_bytes, int n_keys,
                       unsigned long long* hist_dev, void* out, cudaStream_t s);
 cudaError_t trace_occupancy(int precision, bool peel, int block, int* blocks_per_sm, int mode = 0, int anc = 0);
@@ -259,9 +260,12 @@ size_t peel_record_bytes(int precision);
 // node-descent counters of builds compiled with RT_COUNT_DESCENTS=1
 bool descents_counted();
 cudaError_t descent_counts(unsigned long long out[2], bool reset);
-// sort keys of n queued peel-off records: block of 2^bs root cells (x fastest)
-cudaError_t peel_keys(int precision, const void* rec, long long n, int bs, int nbx, int nby, int nbz, uint32_t* key,
-                      int sm_count, cudaStream_t s);
+// n queued peel-off records (with count: min(n, *count), read on the device)
+// sorted by block of 2^bs root cells (x fastest) from rec into out; key: room
+// for n, hist: tile_hist_bytes(nbx * nby * nbz)
+cudaError_t peel_sort(int precision, const void* rec, long long n, const unsigned long long* count, int bs, int nbx,
+                      int nby, int nbz, uint32_t* key, unsigned long long* hist, void* out, int sm_count,
+                      cudaStream_t s);
 // peel-off kernel with the extinction tables of JobDev::ptab
 cudaError_t launch_peel_tab(int precision, const JobDev* jobs_dev, const PeelQueue& q, unsigned long long* work_dev,
                             int n_obs_max, int refill, cudaStream_t s, int anc = 0);

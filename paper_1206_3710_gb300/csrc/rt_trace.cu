@@ -297,6 +297,31 @@ __device__ __forceinline__ unsigned long long claim_slot(unsigned long long* ctr
   return base + (unsigned long long)__popc(m & ((1u << lane) - 1u));
 }
 
+// Work items for the dead lanes of a warp: the item of each lane (at or
+// beyond n: none left).  A warp's first 32 items follow from its number in
+// the grid, the rest come from a counter, and a warp that has seen the end
+// does not ask again.  The counter is one address, its atomics take their
+// turns a few ns apart: by the counter alone a launch of 1e5 packages makes
+// 1.2e4 of them, most for nothing.  state (the warp's, in shared memory): 0
+// nothing taken yet, 1 the end was seen, 2 the warp's own taken.
+__device__ __forceinline__ long long next_work(unsigned long long* counter, long long n, unsigned dead, int leader,
+                                               int lane, int& state) {
+  const int rank = __popc(dead & ((1u << lane) - 1u));
+  const int st = state;
+  __syncwarp();
+  if (st == 0) {
+    // (every lane is dead at a warp's first refill)
+    if (lane == 0) state = 2;
+    return ((long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + rank;
+  }
+  if (st == 1) return n + rank;
+  unsigned long long base = 0ull;
+  if (lane == leader) base = atomicAdd(counter, (unsigned long long)__popc(dead));
+  base = __shfl_sync(0xFFFFFFFFu, base, leader) + 32ull * gridDim.x * (blockDim.x >> 5);
+  if (lane == 0 && (long long)base + __popc(dead) >= n) state = 1;
+  return (long long)base + rank;
+}
+
 // device counters of node descents (a global read of an interior cell's
 // child word each: the 4 B per descent of the roofline unit), kept only in
 // builds compiled with RT_COUNT_DESCENTS=1 (an atomic per descent): [0] the
@@ -572,6 +597,8 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
   __shared__ WarpLedger SL;
   __shared__ ColdState<R> C;
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  __shared__ int s_work[8];  // next_work
+  if (lane == 0) s_work[wid] = 0;
   ledger_init<R>(SL, wid, lane);
   C.job[t] = -1;
   C.crowd[t] = 0u;
@@ -686,10 +713,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
     const unsigned busy = __ballot_sync(FULL, st == ST_TRACE || st == ST_PEEL);
     if (dead != 0u && (__popc(dead) >= refill_thr || busy == 0u)) {
       const int leader = __ffs(dead) - 1;
-      unsigned long long base = 0ull;
-      if (lane == leader) base = atomicAdd(counter, (unsigned long long)__popc(dead));
-      base = __shfl_sync(FULL, base, leader);
-      const long long slot = (long long)base + __popc(dead & ((1u << lane) - 1u));
+      const long long slot = next_work(counter, total - (MODE == 1 ? T.first : 0), dead, leader, lane, s_work[wid]);
       long long gi = MODE == 1 ? T.first + slot : slot;  // package index
       const TRec* rec = nullptr;
       if (MODE == 2 && st == ST_DEAD && slot < total) {
@@ -1442,6 +1466,8 @@ __global__ void __launch_bounds__(256, PeelMinBlocks<R>::value) peel_kernel(cons
   enum { P_DEAD = 0, P_LIVE = 1, P_DONE = 2 };
   __shared__ WarpLedger SL;
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  __shared__ int s_work[8];  // next_work
+  if (lane == 0) s_work[wid] = 0;
   ledger_init<R>(SL, wid, lane);
   // the path above the current leaf (dynamic shared memory, n_anc x 256 words)
   extern __shared__ uint32_t s_anc[];
@@ -1483,10 +1509,7 @@ __global__ void __launch_bounds__(256, PeelMinBlocks<R>::value) peel_kernel(cons
     const unsigned live = __ballot_sync(FULL, st == P_LIVE);
     if (dead != 0u && (__popc(dead) >= refill_thr || live == 0u)) {
       const int leader = __ffs(dead) - 1;
-      unsigned long long base = 0ull;
-      if (lane == leader) base = atomicAdd(work, (unsigned long long)__popc(dead));
-      base = __shfl_sync(FULL, base, leader);
-      const long long gi = (long long)base + __popc(dead & ((1u << lane) - 1u));
+      const long long gi = next_work(work, total, dead, leader, lane, s_work[wid]);
       const bool have = st == P_DEAD && gi < total;
       if (st == P_DEAD && !have) st = P_DONE;
       Geo<R> rg;
@@ -1896,34 +1919,67 @@ __global__ void tile_hist_kernel(const uint32_t* __restrict__ key, long long n, 
       if (sh[k]) atomicAdd(&hist[k], (unsigned long long)sh[k]);
 }
 
-// exclusive prefix sum of hist[0, n) in place, one block
-__global__ void tile_scan_kernel(unsigned long long* hist, int n) {
-  __shared__ unsigned long long part[1024];
-  const int t = threadIdx.x, nt = blockDim.x;
-  const int per = (n + nt - 1) / nt;
-  const int b = t * per, e = min(n, b + per);
-  unsigned long long sum = 0ull;
-  for (int i = b; i < e; ++i) sum += hist[i];
-  part[t] = sum;
-  __syncthreads();
-  for (int off = 1; off < nt; off <<= 1) {
-    const unsigned long long v = t >= off ? part[t - off] : 0ull;
-    __syncthreads();
-    part[t] += v;
-    __syncthreads();
+// Exclusive prefix sums of hist within chunks of SCAN_KEYS, and the chunks'
+// totals; the scatter adds the totals before its key's chunk.  (One block
+// over all 262,144 keys of a peel-off queue took 118 to 400 us.)
+static constexpr int SCAN_KEYS = 4096;
+__global__ void __launch_bounds__(1024) tile_scan_kernel(unsigned long long* __restrict__ hist, int n,
+                                                         unsigned long long* __restrict__ totals) {
+  __shared__ unsigned long long part[32];
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  const int b = blockIdx.x * SCAN_KEYS + 4 * t;
+  unsigned long long v[4], sum = 0ull;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    v[i] = b + i < n ? hist[b + i] : 0ull;
+    sum += v[i];
   }
-  unsigned long long run = part[t] - sum;
-  for (int i = b; i < e; ++i) {
-    const unsigned long long v = hist[i];
-    hist[i] = run;
-    run += v;
+  unsigned long long inc = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long x = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+    if (lane >= o) inc += x;
+  }
+  if (lane == 31) part[wid] = inc;
+  __syncthreads();
+  if (wid == 0) {
+    unsigned long long p = part[lane], q = p;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long x = __shfl_up_sync(0xFFFFFFFFu, q, o);
+      if (lane >= o) q += x;
+    }
+    part[lane] = q - p;
+    if (lane == 31) totals[blockIdx.x] = q;
+  }
+  __syncthreads();
+  unsigned long long run = part[wid] + inc - sum;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if (b + i < n) hist[b + i] = run;
+    run += v[i];
   }
 }
 
 // scatter records to their key's range; lanes of a warp with equal keys
 // take consecutive places with one atomic
 __global__ void tile_scatter_kernel(const uint4* __restrict__ in, const uint32_t* __restrict__ key, long long n,
-                                    int rec_u4, unsigned long long* __restrict__ offs, uint4* __restrict__ out) {
+                                    const unsigned long long* __restrict__ count, int rec_u4, int n_chunks,
+                                    const unsigned long long* __restrict__ totals, unsigned long long* __restrict__ offs,
+                                    uint4* __restrict__ out) {
+  extern __shared__ unsigned long long before[];  // records in the chunks of keys before each
+  if (count) n = min(n, (long long)*count);
+  for (int i = threadIdx.x; i < n_chunks; i += blockDim.x) before[i] = totals[i];
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long run = 0ull;
+    for (int i = 0; i < n_chunks; ++i) {
+      const unsigned long long v = before[i];
+      before[i] = run;
+      run += v;
+    }
+  }
+  __syncthreads();
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long n_up = (n + 31) / 32 * 32;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n_up; i += stride) {
@@ -1936,12 +1992,28 @@ __global__ void tile_scatter_kernel(const uint4* __restrict__ in, const uint32_t
     if (have && lane == leader) base = atomicAdd(&offs[k], (unsigned long long)__popc(peers));
     base = __shfl_sync(peers, base, leader);
     if (have) {
-      const unsigned long long pos = base + __popc(peers & ((1u << lane) - 1u));
+      const unsigned long long pos = before[k / SCAN_KEYS] + base + __popc(peers & ((1u << lane) - 1u));
       const uint4* src = in + i * rec_u4;
       uint4* dst = out + pos * rec_u4;
       for (int w = 0; w < rec_u4; ++w) dst[w] = src[w];
     }
   }
+}
+
+size_t tile_hist_bytes(int n_keys) {
+  return sizeof(unsigned long long) * ((size_t)n_keys + (size_t)(n_keys + SCAN_KEYS - 1) / SCAN_KEYS + 1);
+}
+
+// the scan and scatter of a counting sort whose histogram is in hist
+static cudaError_t sort_by_hist(const void* in, const uint32_t* key, long long n, const unsigned long long* count,
+                                int rec_bytes, int n_keys, unsigned long long* hist, void* out, int grid,
+                                cudaStream_t s) {
+  const int nc = (n_keys + SCAN_KEYS - 1) / SCAN_KEYS;
+  unsigned long long* totals = hist + n_keys;
+  tile_scan_kernel<<<nc, 1024, 0, s>>>(hist, n_keys, totals);
+  tile_scatter_kernel<<<grid, 512, sizeof(unsigned long long) * (size_t)nc, s>>>(
+      static_cast<const uint4*>(in), key, n, count, rec_bytes / 16, nc, totals, hist, static_cast<uint4*>(out));
+  return cudaGetLastError();
 }
 
 cudaError_t tile_sort(const void* in, const uint32_t* key, long long n, int rec_bytes, int n_keys,
@@ -1958,10 +2030,9 @@ cudaError_t tile_sort(const void* in, const uint32_t* key, long long n, int rec_
   const int G = (int)std::min<long long>(want, (long long)sms * 4);
   const size_t shb = n_keys <= 8192 ? sizeof(unsigned int) * (size_t)n_keys : 0;
   tile_hist_kernel<<<G, B, shb, s>>>(key, n, n_keys, hist_dev);
-  tile_scan_kernel<<<1, 1024, 0, s>>>(hist_dev, n_keys);
-  tile_scatter_kernel<<<G, B, 0, s>>>(static_cast<const uint4*>(in), key, n, rec_bytes / 16, hist_dev,
-                                      static_cast<uint4*>(out));
-  return cudaGetLastError();
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  return sort_by_hist(in, key, n, nullptr, rec_bytes, n_keys, hist_dev, out, G, s);
 }
 
 bool descents_counted() { return RT_COUNT_DESCENTS != 0; }
@@ -1979,10 +2050,18 @@ size_t peel_record_bytes(int precision) { return precision == 64 ? sizeof(PeelRe
 
 // sort key of a deferred peel-off record: the block of 2^bs root cells
 // holding the scattering point, x fastest, clamped to the nbx x nby x nbz
-// blocks of the first job's root grid
+// blocks of the first job's root grid; and the keys' histogram
 template <typename R>
-__global__ void peel_key_kernel(const void* __restrict__ rec, long long n, int bs, int nbx, int nby, int nbz,
-                                uint32_t* __restrict__ key) {
+__global__ void __launch_bounds__(512) peel_key_kernel(const void* __restrict__ rec, long long n,
+                                                       const unsigned long long* __restrict__ count, int bs, int nbx,
+                                                       int nby, int nbz, uint32_t* __restrict__ key, int n_keys,
+                                                       unsigned long long* __restrict__ hist) {
+  extern __shared__ unsigned int sh[];
+  const bool use_sh = n_keys <= 8192;
+  if (use_sh)
+    for (int k = threadIdx.x; k < n_keys; k += blockDim.x) sh[k] = 0u;
+  __syncthreads();
+  if (count) n = min(n, (long long)*count);
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     uint4 a;
     uint32_t meta;
@@ -1995,22 +2074,37 @@ __global__ void peel_key_kernel(const void* __restrict__ rec, long long n, int b
       a = __ldg(reinterpret_cast<const uint4*>(&r->cx));
       meta = __ldg(&r->meta);
     }
-    const int sh = (int)(meta & 31u) + bs;
-    const uint32_t bx = min(a.x >> sh, (uint32_t)(nbx - 1));
-    const uint32_t by = min(a.y >> sh, (uint32_t)(nby - 1));
-    const uint32_t bz = min(a.z >> sh, (uint32_t)(nbz - 1));
-    key[i] = bx + (uint32_t)nbx * (by + (uint32_t)nby * bz);
+    const int shf = (int)(meta & 31u) + bs;
+    const uint32_t bx = min(a.x >> shf, (uint32_t)(nbx - 1));
+    const uint32_t by = min(a.y >> shf, (uint32_t)(nby - 1));
+    const uint32_t bz = min(a.z >> shf, (uint32_t)(nbz - 1));
+    const uint32_t k = bx + (uint32_t)nbx * (by + (uint32_t)nby * bz);
+    key[i] = k;
+    if (use_sh) atomicAdd(&sh[k], 1u);
+    else atomicAdd(&hist[k], 1ull);
   }
+  __syncthreads();
+  if (use_sh)
+    for (int k = threadIdx.x; k < n_keys; k += blockDim.x)
+      if (sh[k]) atomicAdd(&hist[k], (unsigned long long)sh[k]);
 }
 
-cudaError_t peel_keys(int precision, const void* rec, long long n, int bs, int nbx, int nby, int nbz, uint32_t* key,
-                      int sm_count, cudaStream_t s) {
+cudaError_t peel_sort(int precision, const void* rec, long long n, const unsigned long long* count, int bs, int nbx,
+                      int nby, int nbz, uint32_t* key, unsigned long long* hist, void* out, int sm_count,
+                      cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  const int B = 256;
-  const int G = (int)std::min<long long>((n + B - 1) / B, (long long)sm_count * 8);
-  if (precision == 64) peel_key_kernel<double><<<G, B, 0, s>>>(rec, n, bs, nbx, nby, nbz, key);
-  else peel_key_kernel<float><<<G, B, 0, s>>>(rec, n, bs, nbx, nby, nbz, key);
-  return cudaGetLastError();
+  const int n_keys = nbx * nby * nbz;
+  cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * (size_t)n_keys, s);
+  if (e != cudaSuccess) return e;
+  const int B = 512;
+  // a count on the device may be far below n: no more blocks than fill the GPU
+  const int G = (int)std::min<long long>((n + B - 1) / B, (long long)sm_count * 4);
+  const size_t shb = n_keys <= 8192 ? sizeof(unsigned int) * (size_t)n_keys : 0;
+  if (precision == 64) peel_key_kernel<double><<<G, B, shb, s>>>(rec, n, count, bs, nbx, nby, nbz, key, n_keys, hist);
+  else peel_key_kernel<float><<<G, B, shb, s>>>(rec, n, count, bs, nbx, nby, nbz, key, n_keys, hist);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  return sort_by_hist(rec, key, n, count, (int)peel_record_bytes(precision), n_keys, hist, out, G, s);
 }
 
 template <typename R, bool TAB>
