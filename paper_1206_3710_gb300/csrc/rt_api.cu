@@ -108,6 +108,9 @@ struct rt_ctx {
     int block = 256, refill = 8, blocks_per_sm = 0;
   } tuned[2][2];
   int cc_major = 0, cc_minor = 0;
+  // blocks per SM of the tracers, by precision, peel-off, mode (0 or 2), path
+  // levels and block size / 32; 0: not asked yet
+  int occ[2][2][2][RT_ANC_MAX + 1][9] = {};
 };
 
 struct rt_grid {
@@ -262,17 +265,19 @@ static PeelQueue make_queue(DevBuf& buf, long long max_records, bool peel, int n
 }
 
 
-// wait for an event with a deadline; the device keeps running on timeout
+// wait for an event with a deadline; the device keeps running on timeout.
+// The first millisecond is polled (a small call's work takes 0.1 to 1 ms, and
+// a sleep of 50 us ends up to 100 us late), then the thread sleeps between
+// polls.
 static int wait_event(cudaEvent_t ev, double timeout_s) {
   const auto t0 = std::chrono::steady_clock::now();
-  int spins = 0;
   for (;;) {
     cudaError_t e = cudaEventQuery(ev);
     if (e == cudaSuccess) return RT_OK;
     if (e != cudaErrorNotReady) return fail(RT_ERR_CUDA, "device error while waiting: %s", cudaGetErrorString(e));
     const double el = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     if (el > timeout_s) return fail(RT_ERR_TIMEOUT, "device work did not finish within %.3f s", timeout_s);
-    if (++spins > 64) std::this_thread::sleep_for(std::chrono::microseconds(50));
+    if (el > 1e-3) std::this_thread::sleep_for(std::chrono::microseconds(50));
   }
 }
 
@@ -1067,15 +1072,18 @@ static int make_cfg(rt_ctx* c, int precision, bool peel, const rt_trace_params* 
   if (cfg->block % 32 || cfg->block > 256 || cfg->block < 32)
     return fail(RT_ERR_INVALID, "block_size must be a multiple of 32 in 32..256");
   cfg->anc = anc;
-  int occ = 0;
-  CK(trace_occupancy(precision, peel, cfg->block, &occ, 0, anc));
-  if (occ < 1) occ = 1;
+  int(*known)[RT_ANC_MAX + 1][9] = c->occ[precision == 64][peel ? 1 : 0];
+  for (int m = 0; m < 2; ++m) {
+    int& o = known[m][anc][cfg->block / 32];
+    if (o > 0) continue;
+    CK(trace_occupancy(precision, peel, cfg->block, &o, 2 * m, anc));
+    if (o < 1) o = 1;
+  }
+  int occ = known[0][anc][cfg->block / 32];
   const int bps = lp->blocks_per_sm > 0 ? lp->blocks_per_sm : (t.set ? t.blocks_per_sm : 0);
   if (bps > 0) occ = std::min(occ, bps);
   cfg->blocks = c->sm_count * occ;
-  int occ2 = 0;
-  CK(trace_occupancy(precision, peel, cfg->block, &occ2, 2, anc));
-  if (occ2 < 1) occ2 = 1;
+  int occ2 = known[1][anc][cfg->block / 32];
   if (bps > 0) occ2 = std::min(occ2, bps);
   cfg->blocks_tiled = c->sm_count * occ2;
   cfg->refill = lp->refill_threshold > 0 ? lp->refill_threshold : (t.set ? t.refill : default_refill(precision, peel));
