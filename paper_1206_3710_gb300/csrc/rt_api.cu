@@ -1066,12 +1066,14 @@ static int path_levels(int n_jobs, const TraceArgs* jobs) {
   return deep ? std::min(d, RT_ANC_MAX) : 0;
 }
 
-static int make_cfg(rt_ctx* c, int precision, bool peel, const rt_trace_params* lp, int anc, LaunchCfg* cfg) {
+static int make_cfg(rt_ctx* c, int precision, bool peel, const rt_trace_params* lp, int anc, int n_jobs,
+                    LaunchCfg* cfg) {
   const rt_ctx::Tuned& t = c->tuned[precision == 64][peel ? 1 : 0];
   cfg->block = lp->block_size > 0 ? lp->block_size : (t.set ? t.block : 256);
   if (cfg->block % 32 || cfg->block > 256 || cfg->block < 32)
     return fail(RT_ERR_INVALID, "block_size must be a multiple of 32 in 32..256");
   cfg->anc = anc;
+  cfg->ev_batch = n_jobs > 1 ? 16 : 12;
   int(*known)[RT_ANC_MAX + 1][9] = c->occ[precision == 64][peel ? 1 : 0];
   for (int m = 0; m < 2; ++m) {
     int& o = known[m][anc][cfg->block / 32];
@@ -1284,7 +1286,7 @@ static int run_jobs(rt_ctx* c, int n_jobs, const TraceArgs* jobs, rt_ledger* led
   const bool poly = n_jobs == 1 && jobs[0].prm->poly_group > 1;
   const PeelQueue q = make_queue(c->peel_q, c->peel_q_max, peel && !poly, n_jobs, total, precision, counter + 1);
   LaunchCfg cfg;
-  rc = make_cfg(c, precision, peel, launch_prm, path_levels(n_jobs, jobs), &cfg);
+  rc = make_cfg(c, precision, peel, launch_prm, path_levels(n_jobs, jobs), n_jobs, &cfg);
   if (rc) return rc;
   bool hits = false;
   for (int j = 0; j < n_jobs; ++j) hits = hits || jobs[j].prm->hits_dev != nullptr;
@@ -2065,7 +2067,7 @@ extern "C" int rt_batch_create(rt_ctx* ctx, int n_jobs, const rt_job* jobs, rt_b
   e = cudaStreamSynchronize(b->cap);
   if (e != cudaSuccess) return bail(fail(RT_ERR_CUDA, "rt_batch_create: %s", cudaGetErrorString(e)));
   LaunchCfg cfg;
-  rc = make_cfg(ctx, precision, peel, jobs[0].params, path_levels(n_jobs, args.data()), &cfg);
+  rc = make_cfg(ctx, precision, peel, jobs[0].params, path_levels(n_jobs, args.data()), n_jobs, &cfg);
   if (rc) return bail(rc);
   const PeelQueue q = make_queue(b->peel_q, ctx->peel_q_max, peel, n_jobs, total, precision, counter + 1);
   // capture: zero every job's outputs and the ledgers, run the tracer and

@@ -60,6 +60,16 @@ struct Num<float> {
   // offset f moved by t along d, kept in [0, 1]
   static __device__ __forceinline__ float moved01(float f, float t, float d) { return __saturatef(fmaf(t, d, f)); }
   static __device__ __forceinline__ float min_(float a, float b) { return fminf(a, b); }
+  // comparisons of non-negative numbers, and of a direction component with 0
+  static __device__ __forceinline__ bool same(float a, float b) { return a == b; }
+  static __device__ __forceinline__ bool ge(float a, float b) { return a >= b; }
+  static __device__ __forceinline__ bool pos(float a) { return a > 0.0f; }
+  static __device__ __forceinline__ bool finite(float a) { return a < CUDART_INF_F; }
+  static __device__ __forceinline__ bool not_neg(float d) { return d >= 0.0f; }
+  static __device__ __forceinline__ bool above(float f, float h) { return f > h; }
+  static __device__ __forceinline__ float one_if(uint32_t b) { return (float)b; }
+  // v 2^-l, 0 <= l <= 126
+  static __device__ __forceinline__ float down(float v, int l) { return v * pow2m(l); }
   // 2^-l for 0 <= l <= 126, exact
   static __device__ __forceinline__ float pow2m(int l) { return __int_as_float((127 - l) << 23); }
   static __device__ __forceinline__ float leaf_rho(uint32_t w, double) { return __uint_as_float(w); }
@@ -80,9 +90,25 @@ struct Num<double> {
   static __device__ __forceinline__ double uni(uint32_t x) { return ((double)x + 0.5) * 2.3283064365386963e-10; }
   static __device__ __forceinline__ double log_(double x) { return log(x); }
   static __device__ __forceinline__ double expm1_(double x) { return expm1(x); }
+  // q = 1 - exp(-x), e = 1 - q: Taylor series below 1/8 (relative remainder
+  // below 3e-17 with the terms to x^10, below 2^-9 with those to x^5), exp
+  // above
   static __device__ __forceinline__ void absorb_pair(double x, double& q, double& e) {
-    if (x < 0.125) {
-      q = -expm1(-x);
+    const int hi = __double2hiint(x);
+    if (hi < 0x3FC00000) {
+      double s = 1.0 / 120.0;
+      if (hi >= 0x3F600000) {
+        s = 1.0 / 3628800.0;
+        s = fma(-x, s, 1.0 / 362880.0);
+        s = fma(-x, s, 1.0 / 40320.0);
+        s = fma(-x, s, 1.0 / 5040.0);
+        s = fma(-x, s, 1.0 / 720.0);
+        s = fma(-x, s, 1.0 / 120.0);
+      }
+      s = fma(-x, s, 1.0 / 24.0);
+      s = fma(-x, s, 1.0 / 6.0);
+      s = fma(-x, s, 0.5);
+      q = fma(-x, x * s, x);
       e = 1.0 - q;
     } else {
       e = exp(-x);
@@ -97,12 +123,34 @@ struct Num<double> {
   static __device__ __forceinline__ double ldexp_(double x, int e) { return ldexp(x, e); }
   static __device__ __forceinline__ void sincos2pi(double u, double* s, double* c) { sincospi(2.0 * u, s, c); }
   static __device__ __forceinline__ double inf() { return CUDART_INF; }
-  static __device__ __forceinline__ double ahead(double d) { return d > 0.0 ? 1.0 : 0.0; }
+  // The FP64 pipe has two lanes per SM and clock, the integer pipes 128, and
+  // non-negative doubles order like their bit patterns: comparisons, selects,
+  // clamps and powers of two are taken from the bits (the results are those of
+  // the FP64 operations; a NaN, from inf * 0, ranks above inf).
+  static __device__ __forceinline__ unsigned long long b(double v) {
+    return (unsigned long long)__double_as_longlong(v);
+  }
+  static __device__ __forceinline__ double ahead(double d) {
+    return __hiloint2double(__double2hiint(d) < 0 ? 0 : 0x3FF00000, 0);
+  }
   static __device__ __forceinline__ double moved01(double f, double t, double d) {
     const double v = fma(t, d, f);
-    return v < 0.0 ? 0.0 : (v > 1.0 ? 1.0 : v);
+    const int hi = __double2hiint(v);
+    return hi < 0 ? 0.0 : (hi >= 0x3FF00000 ? 1.0 : v);
   }
-  static __device__ __forceinline__ double min_(double a, double b) { return fmin(a, b); }
+  static __device__ __forceinline__ double min_(double x, double y) { return b(x) < b(y) ? x : y; }
+  static __device__ __forceinline__ bool same(double x, double y) { return b(x) == b(y); }
+  static __device__ __forceinline__ bool ge(double x, double y) { return b(x) >= b(y); }
+  static __device__ __forceinline__ bool pos(double x) { return b(x) != 0ull; }
+  static __device__ __forceinline__ bool finite(double x) { return __double2hiint(x) < 0x7FF00000; }
+  static __device__ __forceinline__ bool not_neg(double d) { return __double2hiint(d) >= 0 || (b(d) << 1) == 0ull; }
+  static __device__ __forceinline__ bool above(double f, double h) { return b(f) > b(h); }
+  static __device__ __forceinline__ double one_if(uint32_t u) { return __hiloint2double(u ? 0x3FF00000 : 0, 0); }
+  static __device__ __forceinline__ double down(double v, int l) {
+    const int hi = __double2hiint(v);
+    if ((hi >> 20) > l) return __hiloint2double(hi - (l << 20), __double2loint(v));
+    return b(v) == 0ull ? v : v * pow2m(l);
+  }
   static __device__ __forceinline__ double pow2m(int l) { return __longlong_as_double((long long)(1023 - l) << 52); }
   static __device__ __forceinline__ double leaf_rho(uint32_t, double r64) { return r64; }
   static __device__ __forceinline__ double load_rho64(const double* p, uint32_t i) { return __ldg(p + i); }
@@ -172,7 +220,7 @@ struct GridRegs {
 // a point on a face belongs to the child the direction points into
 template <typename R>
 __device__ __forceinline__ uint32_t upper_half(R f, R d) {
-  return (f > R(0.5)) | ((f == R(0.5)) & (d >= R(0)));
+  return Num<R>::above(f, R(0.5)) | (Num<R>::same(f, R(0.5)) & Num<R>::not_neg(d));
 }
 
 // one level of descent below a refined node word w at cursor level k
@@ -185,9 +233,9 @@ __device__ __forceinline__ void descend_step(Geo<R>& g, Cursor& cur, uint32_t w,
   const uint32_t ol = ((g.cx >> sh) & 1u) | (((g.cy >> sh) & 1u) << 1) | (((g.cz >> sh) & 1u) << 2);
   const uint32_t bx = upper_half(g.fx, dx), by = upper_half(g.fy, dy), bz = upper_half(g.fz, dz);
   if (!by_lattice) {
-    g.fx = R(2) * g.fx - R(bx);
-    g.fy = R(2) * g.fy - R(by);
-    g.fz = R(2) * g.fz - R(bz);
+    g.fx = R(2) * g.fx - Num<R>::one_if(bx);
+    g.fy = R(2) * g.fy - Num<R>::one_if(by);
+    g.fz = R(2) * g.fz - Num<R>::one_if(bz);
     g.cx = 2u * g.cx + bx;
     g.cy = 2u * g.cy + by;
     g.cz = 2u * g.cz + bz;
@@ -282,73 +330,10 @@ __device__ __forceinline__ bool place_root(const GridRegs& G, Geo<R>& g, Cursor&
   return true;
 }
 
-// exit distance (leaf-local units) and axis; ties -> lowest axis.  Axes with
-// d == 0 give NaN or inf and are never selected.
-template <typename R>
-__device__ __forceinline__ R exit_dist(const Geo<R>& g, R dx, R dy, R dz, R ix, R iy, R iz, int& axis) {
-  const R tx = (dx > R(0) ? R(1) - g.fx : g.fx) * ix;
-  const R ty = (dy > R(0) ? R(1) - g.fy : g.fy) * iy;
-  const R tz = (dz > R(0) ? R(1) - g.fz : g.fz) * iz;
-  R t = Num<R>::inf();
-  int a = -1;
-  if (tx < t) { t = tx; a = 0; }
-  if (ty < t) { t = ty; a = 1; }
-  if (tz < t) { t = tz; a = 2; }
-  axis = a;
-  return t;
-}
-
-template <typename R>
-__device__ __forceinline__ R clamp01(R v) {
-  return v < R(0) ? R(0) : (v > R(1) ? R(1) : v);
-}
-
-// Cross the exit face on axis a; aim the cursor at the neighbour (the
-// sibling in the same octet or the root-level neighbour with one load,
-// otherwise a descent from the sibling of the deepest stored ancestor the
-// neighbour does not share, or from the root cell: neighbour_start).  False
-// when the package leaves the root grid.  Written with selects only: lanes
-// crossing different axes do not diverge.  `moved` gets the bits of the lattice coordinate on axis a
-// that changed (bit l + s set: the crossing left a block of 2^s cells of
-// level l on that axis, e.g. a tile).
-template <typename R>
-__device__ __forceinline__ bool advance(const GridRegs& G, Geo<R>& g, Cursor& cur, int a, R t, R dx, R dy, R dz,
-                                        uint32_t& moved, AncPath& P) {
-  const bool a0 = a == 0, a1 = a == 1;
-  const R da = a0 ? dx : (a1 ? dy : dz);
-  const bool plus = da > R(0);
-  const R fnew = plus ? R(0) : R(1);
-  const R nfx = clamp01(g.fx + t * dx), nfy = clamp01(g.fy + t * dy), nfz = clamp01(g.fz + t * dz);
-  g.fx = a0 ? fnew : nfx;
-  g.fy = a1 ? fnew : nfy;
-  g.fz = (!a0 && !a1) ? fnew : nfz;
-  const uint32_t cold = a0 ? g.cx : (a1 ? g.cy : g.cz);
-  const uint32_t cnew = plus ? cold + 1u : cold - 1u;
-  g.cx = a0 ? cnew : g.cx;
-  g.cy = a1 ? cnew : g.cy;
-  g.cz = (!a0 && !a1) ? cnew : g.cz;
-  moved = cold ^ cnew;
-  // only axis a moved: inside while its root coordinate stays below the
-  // root grid's size (a step below 0 wraps to a huge unsigned value)
-  const bool inside = (cnew >> g.lev) < (a0 ? G.rx : (a1 ? G.ry : G.rz));
-  neighbour_start(G, g.lev, g.idx, g.cx, g.cy, g.cz, a, plus, moved, P, cur);
-  return inside;
-}
-template <typename R>
-__device__ __forceinline__ bool advance(const GridRegs& G, Geo<R>& g, Cursor& cur, int a, R t, R dx, R dy, R dz,
-                                        uint32_t& moved) {
-  AncPath P = no_path();
-  return advance(G, g, cur, a, t, dx, dy, dz, moved, P);
-}
-template <typename R>
-__device__ __forceinline__ bool advance(const GridRegs& G, Geo<R>& g, Cursor& cur, int a, R t, R dx, R dy, R dz) {
-  uint32_t moved;
-  return advance(G, g, cur, a, t, dx, dy, dz, moved);
-}
-
-// advance() for a direction along axis a (the other two components zero):
-// the offsets on the other axes do not move, so only axis a is updated
-// (the same results as advance() with that direction)
+// cross_face() for a direction along axis a (the other two components
+// zero): the offsets on the other axes do not move, so only axis a is
+// updated (the same results as cross_face() with that direction).  False
+// when the package leaves the root grid.
 template <typename R>
 __device__ __forceinline__ bool advance_axis(const GridRegs& G, Geo<R>& g, Cursor& cur, int a, bool plus,
                                              AncPath& P) {
@@ -385,16 +370,22 @@ __device__ __forceinline__ Exit<R> exit_face(const Geo<R>& g, R dx, R dy, R dz, 
   E.sz = Num<R>::ahead(dz);
   const R tx = fabs(E.sx - g.fx) * ix, ty = fabs(E.sy - g.fy) * iy, tz = fabs(E.sz - g.fz) * iz;
   E.t = Num<R>::min_(Num<R>::min_(tx, ty), tz);
-  E.x = tx == E.t;
-  E.y = !E.x && ty == E.t;
+  E.x = Num<R>::same(tx, E.t);
+  E.y = !E.x && Num<R>::same(ty, E.t);
   return E;
 }
 
-// Move by t from leaf idx and, with go, cross that face (as advance(), which
-// takes the axis as a number): the offsets move and stay in [0, 1], the
-// offset on the crossing axis becomes that of the neighbour's near face, the
-// cursor aims at the neighbour.  Without go the cursor and the lattice
-// coordinates stay.  False when the package leaves the root grid.
+// Move by t from leaf idx and, with go, cross that face: the offsets move and
+// stay in [0, 1], the offset on the crossing axis becomes that of the
+// neighbour's near face, and the cursor aims at the neighbour (the sibling
+// in the same octet or the root-level neighbour with one load, otherwise a
+// descent from the sibling of the deepest stored ancestor the neighbour does
+// not share, or from the root cell).  Without go the cursor and the lattice
+// coordinates stay.  False when the package leaves the root grid.  Written
+// with selects only: lanes crossing different axes do not diverge.  `moved`
+// gets the bits of the lattice coordinate on the crossing axis that changed
+// (bit l + s set: the crossing left a block of 2^s cells of level l on that
+// axis, e.g. a tile).
 template <typename R>
 __device__ __forceinline__ bool cross_face(const GridRegs& G, Geo<R>& g, Cursor& cur, uint32_t idx, const Exit<R>& E,
                                            R t, bool go, R dx, R dy, R dz, uint32_t& moved, AncPath& P) {
@@ -405,7 +396,7 @@ __device__ __forceinline__ bool cross_face(const GridRegs& G, Geo<R>& g, Cursor&
   g.fx = ex ? fnew : nx;
   g.fy = ey ? fnew : ny;
   g.fz = ez ? fnew : nz;
-  const uint32_t sgn = sa > R(0) ? 1u : 0xFFFFFFFFu;
+  const uint32_t sgn = Num<R>::pos(sa) ? 1u : 0xFFFFFFFFu;
   const uint32_t cold = ex ? g.cx : (ey ? g.cy : g.cz);
   const uint32_t cnew = cold + sgn;
   g.cx = ex ? cnew : g.cx;
@@ -429,6 +420,14 @@ __device__ __forceinline__ bool cross_face(const GridRegs& G, Geo<R>& g, Cursor&
     cur.k = near ? g.lev : 0;
   }
   return inside;
+}
+
+template <typename R>
+__device__ __forceinline__ bool cross_face(const GridRegs& G, Geo<R>& g, Cursor& cur, uint32_t idx, const Exit<R>& E,
+                                           R dx, R dy, R dz) {
+  AncPath P = no_path();
+  uint32_t moved;
+  return cross_face(G, g, cur, idx, E, E.t, true, dx, dy, dz, moved, P);
 }
 
 template <typename R>

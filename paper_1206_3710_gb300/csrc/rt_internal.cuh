@@ -232,6 +232,7 @@ struct LaunchCfg {
   int blocks;        // grid of the untiled and emission launches
   int refill;
   int blocks_tiled;  // grid of the tiled rounds (their tracer is sized for fewer blocks per SM)
+  int ev_batch = 12; // lanes with an event that a warp of an untiled launch serves together
   int anc = 0;       // levels of the stored path per lane (0..RT_ANC_MAX): the grids' depth
 };
 

@@ -191,9 +191,9 @@ __global__ void __launch_bounds__(256) poly_kernel(const JobDev* __restrict__ jo
         continue;
       }
       settle_leaf(g, cur, w, r64);
-      int a;
-      const R tx = exit_dist(g, dx, dy, dz, ix, iy, iz, a);
-      if (ncross >= step_limit || a < 0) {
+      const Exit<R> E = exit_face(g, dx, dy, dz, ix, iy, iz);
+      const R tx = E.t;
+      if (ncross >= step_limit || !Num<R>::finite(tx)) {
         R s = R(0);
 #pragma unroll
         for (int j = 0; j < F; ++j) s += W[j];
@@ -233,9 +233,9 @@ __global__ void __launch_bounds__(256) poly_kernel(const JobDev* __restrict__ jo
       if (!per_bin && absb && dsum > R(0)) red_acc(absb + g.idx, widen(dsum));
       ncross += tseg > R(0) ? 1u : 0u;
       if (ev) {
-        g.fx = clamp01(g.fx + tseg * dx);
-        g.fy = clamp01(g.fy + tseg * dy);
-        g.fz = clamp01(g.fz + tseg * dz);
+        g.fx = Num<R>::moved01(g.fx, tseg, dx);
+        g.fy = Num<R>::moved01(g.fy, tseg, dy);
+        g.fz = Num<R>::moved01(g.fz, tseg, dz);
         cur.pending = g.idx;
         cur.k = g.lev;
         nscat += 1;
@@ -273,12 +273,12 @@ __global__ void __launch_bounds__(256) poly_kernel(const JobDev* __restrict__ jo
                 continue;
               }
               settle_leaf(g2, c2, w2, q64);
-              int a2;
-              const R t2 = exit_dist(g2, kx, ky, kz, jx, jy, jz, a2);
-              if (a2 < 0) break;
+              const Exit<R> E2 = exit_face(g2, kx, ky, kz, jx, jy, jz);
+              const R t2 = E2.t;
+              if (!Num<R>::finite(t2)) break;
               col += g2.rho * Num<R>::pow2m(g2.lev) * t2;
               u_pcross += t2 > R(0) ? 1u : 0u;
-              if (!advance(G, g2, c2, a2, t2, kx, ky, kz)) break;
+              if (!cross_face(G, g2, c2, g2.idx, E2, kx, ky, kz)) break;
             }
             const R mu_o = dx * kx + dy * ky + dz * kz;
             const long long pix0 = ((long long)fv) * O.nx + (long long)fu;
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(256) poly_kernel(const JobDev* __restrict__ jo
           }
         }
         tau = -Num<R>::log_(Num<R>::uni(S.word()));
-      } else if (!advance(G, g, cur, a, tx, dx, dy, dz)) {
+      } else if (!cross_face(G, g, cur, g.idx, E, dx, dy, dz)) {
         R s = R(0);
 #pragma unroll
         for (int j = 0; j < F; ++j) s += W[j];

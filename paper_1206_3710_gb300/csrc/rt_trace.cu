@@ -153,13 +153,14 @@ __device__ __forceinline__ unsigned long long sum_lanes_u32(unsigned m, uint32_t
   return (unsigned long long)a + ((unsigned long long)b << 16);
 }
 
-// The slot of the job that all calling lanes (mask m) book to; -1: they book
-// to several jobs, or to one without a slot.
-__device__ __forceinline__ int common_slot(const WarpLedger& SL, unsigned m, int job, int wid) {
-  const int j0 = __shfl_sync(m, job, __ffs(m) - 1);
-  const bool same = __all_sync(m, job == j0);
+// The slot of the job that all calling lanes (mask m) book entry i to; -1:
+// they book to several jobs or entries (lanes of different call sites can
+// meet where the compiler shares their code), or to a job without a slot.
+__device__ __forceinline__ int common_slot(const WarpLedger& SL, unsigned m, int job, int i, int wid) {
+  const int key = job * 32 + i;
+  const bool same = __all_sync(m, key == __shfl_sync(m, key, __ffs(m) - 1));
   if (!same) return -1;
-  return SL.tag[0][wid] == j0 ? 0 : (SL.tag[1][wid] == j0 ? 1 : -1);
+  return SL.tag[0][wid] == job ? 0 : (SL.tag[1][wid] == job ? 1 : -1);
 }
 
 // Bookings come in batches: the lanes that book together are summed in
@@ -171,7 +172,7 @@ __device__ __forceinline__ void book_d(WarpLedger& SL, const JobDev* jobs, int j
   if (v == R(0)) return;
   if (sizeof(R) == 4) {
     const unsigned m = __activemask();
-    const int sl = common_slot(SL, m, job, wid);
+    const int sl = common_slot(SL, m, job, i, wid);
     if (sl >= 0) {
       const unsigned long long q = sum_lanes_u64(m, to_fixed((float)v, SL.shift[sl][wid]));
       if ((threadIdx.x & 31) == (unsigned)(__ffs(m) - 1)) atomicAdd(&SL.d[sl][i][wid], q);
@@ -190,7 +191,7 @@ __device__ __forceinline__ void book_d(WarpLedger& SL, const JobDev* jobs, int j
 __device__ __forceinline__ void book_u(WarpLedger& SL, const JobDev* jobs, int job, int wid, int i, uint32_t v) {
   if (v == 0u) return;
   const unsigned m = __activemask();
-  const int sl = common_slot(SL, m, job, wid);
+  const int sl = common_slot(SL, m, job, i, wid);
   if (sl >= 0) {
     const unsigned long long q = sum_lanes_u32(m, v);
     if ((threadIdx.x & 31) == (unsigned)(__ffs(m) - 1)) atomicAdd(&SL.u[sl][i][wid], q);
@@ -270,19 +271,18 @@ enum { EV_NONE = 0, EV_IDLE, EV_INTERACT, EV_ESCAPE, EV_CUT, EV_KILL, EV_DEGEN, 
 // waiting events together.  Each visit to the event code costs the warp the
 // same whatever the number of lanes it serves, so serving one event per
 // visit (batch 1) spends most issue slots on lanes that do nothing.
+// The batch is the launch's: 12, and 16 for the tiled rounds and for launches
+// of several jobs (small models, whose packages live for few passes).
 // Batches of 8 / 10 / 12 / 16 / 20 lanes: the tiled rounds of a 256^3 cloud
 // step (4e7 packages) 180.8 / 167.8 / 158.9 / 153.4 / 156.1 ms, where most
 // events write a record; the untiled 128^3 cloud (4e6 packages) 5.17 / 5.08 /
 // 5.11 / 5.35 / 5.76 ms, a batched launch of 16 models 8.00 / 7.80 / 7.69 /
 // 7.49 / 7.80 ms.
-#ifndef RT_EV_BATCH
-#define RT_EV_BATCH 12
-#endif
-#ifndef RT_EV_BATCH_TILED
-#define RT_EV_BATCH_TILED 16
-#endif
+// the marches: 8 / 12 / 16 lanes, 256^3 cloud step 138.7 / 138.5 / 135.5 ms,
+// tabulated maps 3.44 / 3.34 / 3.23 ms, FP64 map 3.43 / 3.33 / 3.32 ms, deep
+// cloud 6.41 / 6.54 / 6.46 ms
 #ifndef RT_PEEL_EV_BATCH
-#define RT_PEEL_EV_BATCH 8
+#define RT_PEEL_EV_BATCH 16
 #endif
 // counter slot for each calling lane with one atomic per group of lanes
 // that arrive together (the tile-record and peel-off queues have one
@@ -291,6 +291,9 @@ __device__ __forceinline__ unsigned long long claim_slot(unsigned long long* ctr
   const unsigned m = __activemask();
   const int lane = threadIdx.x & 31;
   const int leader = __ffs(m) - 1;
+  // (lanes that claim from the two queues can meet here)
+  const unsigned long long c = (unsigned long long)ctr;
+  if (!__all_sync(m, c == __shfl_sync(m, c, leader))) return atomicAdd(ctr, 1ull);
   unsigned long long base = 0ull;
   if (lane == leader) base = atomicAdd(ctr, (unsigned long long)__popc(m));
   base = __shfl_sync(m, base, leader);
@@ -590,7 +593,8 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
                                                                          int n_items,
                                                                          unsigned long long* __restrict__ counter,
                                                                          long long total, int refill_thr,
-                                                                         PeelQueue Q, TileRun T, int n_anc) {
+                                                                         int ev_batch, PeelQueue Q, TileRun T,
+                                                                         int n_anc) {
   typedef TileIO<R, LEVELS || SPLIT> IO;
   typedef typename IO::Rec TRec;
   const unsigned FULL = 0xFFFFFFFFu;
@@ -986,7 +990,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
     }
 
     // ------------------------------------------------------------- fast path
-    // Step cells until RT_EV_BATCH lanes of the warp have met an event, or
+    // Step cells until ev_batch lanes of the warp have met an event, or
     // none steps any more.  One node word per lane and pass: a refined node
     // advances the descent by a level, a leaf gets one segment (Sect. 2.3)
     // and a face crossing.  The word of the next node is fetched as soon as
@@ -1014,13 +1018,13 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
           }
           if (tr && ncross >= step_limit) {
             ev = EV_KILL;
-          } else if (!(tx < Num<R>::inf())) {
+          } else if (!Num<R>::finite(tx)) {
             ev = EV_DEGEN;  // cannot happen for |d| = 1
           } else if (SPLIT && tr && lvs != plev) {
             ev = EV_SPLIT;  // entered a grid of another level: resample first
           } else {
             const int lev = g.lev;
-            const R kl = kext * g.rho * Num<R>::pow2m(lev);  // extinction per local unit
+            const R kl = Num<R>::down(kext * g.rho, lev);  // extinction per local unit
             // continuous: the free path is drawn in scattering optical depth
             // (the weight decays by the absorbed fraction along the segment);
             // analog: in extinction optical depth
@@ -1031,7 +1035,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
             double* const dep_to = absb;
             if (!tr) {
               taup += kl * tx;
-              npeel += tx > R(0) ? 1u : 0u;
+              npeel += Num<R>::pos(tx) ? 1u : 0u;
             }
             if (inside_event) {
               tseg = tau / kev;
@@ -1044,7 +1048,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
             } else {
               uint32_t moved;
               const int ax = E.x ? 0 : (E.y ? 1 : 2);
-              if (!advance(G, g, cur, ax, tx, dx, dy, dz, moved, P)) {
+              if (!cross_face(G, g, cur, leaf, E, tx, true, dx, dy, dz, moved, P)) {
                 ev = EV_ESCAPE;
               } else {
                 fetch_node();
@@ -1140,25 +1144,26 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
         }
       }
       const Exit<R> E = exit_face(g, dx, dy, dz, ix, iy, iz);
-      const R kl = kext * Num<R>::leaf_rho(w, r64) * Num<R>::pow2m(lev);  // extinction per local unit
+      const R kl = Num<R>::down(kext * Num<R>::leaf_rho(w, r64), lev);  // extinction per local unit
       // continuous: the free path is drawn in scattering optical depth (the
       // weight decays by the absorbed fraction along the segment); analog:
       // in extinction optical depth.  tau > 0, so an interaction has kev > 0
       const R kev = EST == RT_EST_CONTINUOUS ? alb * kl : kl;
       const R tev = kev * E.t;
-      const bool hit = tev >= tau;
+      const bool hit = Num<R>::ge(tev, tau);
       double* const dep_to = absb;
       R tseg = E.t, x = R(0), ex = R(1);
       if (EST == RT_EST_CONTINUOUS) {
         const R ka = kl - kev;
         x = ka * tseg;
-        if (hit || !Num<R>::thin_seg(x) || !(kl >= thin_lim)) {
+        const bool thin = sizeof(R) == 4 && !(kl >= thin_lim);
+        if (hit || !Num<R>::thin_seg(x) || thin) {
           if (hit) {
             tseg = tau / kev;
             x = ka * tseg;
           }
           if (!Num<R>::thin_seg(x)) ex = Num<R>::exp_(-x);
-          if (!(kl >= thin_lim) && tseg > R(0)) {
+          if (thin && tseg > R(0)) {
             // a near-vacuum cell: its extinction per unit length is below
             // the f32 normal range, so the deposit is taken from the f64
             // density in the thin limit q = x (x < 1e-38; the weight and
@@ -1181,7 +1186,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
       uint32_t moved;
       const bool inside = cross_face(G, g, cur, leaf, E, tseg, !hit, dx, dy, dz, moved, P);
       ev = hit ? EV_INTERACT : (inside ? EV_NONE : EV_ESCAPE);
-      if (!(E.t < Num<R>::inf())) ev = EV_DEGEN;  // cannot happen for |d| = 1
+      if (!Num<R>::finite(E.t)) ev = EV_DEGEN;  // cannot happen for |d| = 1
       if (ev == EV_NONE) {
         fetch_node();
         if (MODE == 2 && (moved >> (lev + T.tsh)) != 0u) ev = EV_TILE;  // entered another tile: next round
@@ -1205,7 +1210,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
         Num<R>::absorb_given(x, ex, q, e);
         const R dep = W * q;
         W = W * e;
-        if (dep > R(0) && (sizeof(R) != 4 || kl >= R(FLT_MIN))) {
+        if (Num<R>::pos(dep) && (sizeof(R) != 4 || kl >= R(FLT_MIN))) {
           pkt_abs += dep;
           if (GROUPED && ncross < C.crowd[t]) {
             if (dep_to || (HITS && hitp))
@@ -1218,10 +1223,10 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
         }
       }
       tau = hit ? R(0) : tau - tev;
-      ncross += tseg > R(0) ? 1u : 0u;
+      ncross += Num<R>::pos(tseg) ? 1u : 0u;
     };
     // every lane that leaves EV_NONE in the loop waits with an event
-    const int stay = max(0, __popc(__ballot_sync(FULL, ev == EV_NONE)) - (MODE == 2 ? RT_EV_BATCH_TILED : RT_EV_BATCH));
+    const int stay = max(0, __popc(__ballot_sync(FULL, ev == EV_NONE)) - ev_batch);
     if (RT_TRACE_ONLY_LOOP && (!PEEL || __ballot_sync(FULL, st == ST_PEEL) == 0u)) {
       // packages fresh from a point source or a beam
       for (int i = 0; i < 64 && __any_sync(FULL, ev == EV_NONE && ncross < C.crowd[t]); ++i)
@@ -1442,6 +1447,8 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
 // the extinction optical depth, and adds W p_HG e^{-tau} to its pixel.
 // Persistent warps refill finished lanes from a global counter.
 // ------------------------------------------------------------------------
+// Blocks per SM: 5 (48 registers), with the stored path 4 (64: the deep cloud
+// 6.16 against 6.41 ms, the 256^3 cloud without it 140.3 against 138.8 ms)
 #ifndef RT_PEEL_MIN_BLOCKS
 #define RT_PEEL_MIN_BLOCKS 5
 #endif
@@ -1451,13 +1458,13 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
 #ifndef RT_PEEL_OBS_MAJOR
 #define RT_PEEL_OBS_MAJOR 1
 #endif
-template <typename R>
+template <typename R, bool PATH>
 struct PeelMinBlocks {
-  static constexpr int value = sizeof(R) == 4 ? RT_PEEL_MIN_BLOCKS : 2;
+  static constexpr int value = sizeof(R) == 4 ? RT_PEEL_MIN_BLOCKS - (PATH ? 1 : 0) : 2;
 };
 
 template <typename R, bool TAB, bool PATH = false>
-__global__ void __launch_bounds__(256, PeelMinBlocks<R>::value) peel_kernel(const JobDev* __restrict__ jobs,
+__global__ void __launch_bounds__(256, PeelMinBlocks<R, PATH>::value) peel_kernel(const JobDev* __restrict__ jobs,
                                                                            PeelQueue Q,
                                                                            unsigned long long* __restrict__ work,
                                                                            int n_obs_max, int refill_thr,
@@ -1618,6 +1625,7 @@ __global__ void __launch_bounds__(256, PeelMinBlocks<R>::value) peel_kernel(cons
             settle_leaf(g, cur, w, r64);
             int a;
             R tx;
+            Exit<R> E;
             if (AX >= 0) {
               const R f = AX == 0 ? g.fx : (AX == 1 ? g.fy : g.fz);
               tx = PL ? R(1) - f : f;
@@ -1628,19 +1636,21 @@ __global__ void __launch_bounds__(256, PeelMinBlocks<R>::value) peel_kernel(cons
               tx = pplus ? R(1) - f : f;
               a = pax;
             } else {
-              tx = exit_dist(g, dx, dy, dz, ix, iy, iz, a);
+              E = exit_face(g, dx, dy, dz, ix, iy, iz);
+              tx = E.t;
+              a = E.x ? 0 : (E.y ? 1 : 2);
             }
             uint32_t moved;
-            if (a < 0) {
+            if (AX < 0 && !Num<R>::finite(tx)) {
               ev = EV_CUT;  // cannot happen for |k| = 1
             } else {
-              taup += kext * g.rho * Num<R>::pow2m(g.lev) * tx;
-              npeel += tx > R(0) ? 1u : 0u;
-              if (taup > tau_cut) {
+              taup += Num<R>::down(kext * g.rho, g.lev) * tx;
+              npeel += Num<R>::pos(tx) ? 1u : 0u;
+              if (!Num<R>::ge(tau_cut, taup)) {
                 ev = EV_CUT;
               } else if (!(AX >= 0     ? advance_axis(G, g, cur, AX, PL, P)
                            : pax >= 0 ? advance_axis(G, g, cur, a, pplus, P)
-                                      : advance(G, g, cur, a, tx, dx, dy, dz, moved, P))) {
+                                      : cross_face(G, g, cur, g.idx, E, tx, true, dx, dy, dz, moved, P))) {
                 ev = EV_ESCAPE;
               } else if (TAB && cur.k == 0) {
                 const JobDev& J = jobs[job];
@@ -1759,9 +1769,9 @@ __global__ void walk_kernel(const JobDev* __restrict__ job, long long n_rays, co
       continue;
     }
     settle_leaf(g, cur, w, r64);
-    int a;
-    const R t = exit_dist(g, dx, dy, dz, ix, iy, iz, a);
-    if (a < 0) break;
+    const Exit<R> E = exit_face(g, dx, dy, dz, ix, iy, iz);
+    const R t = E.t;
+    if (!Num<R>::finite(t)) break;
     if (t > R(0)) {
       if (k < max_seg) {
         cells[r * max_seg + k] = g.idx;
@@ -1769,7 +1779,7 @@ __global__ void walk_kernel(const JobDev* __restrict__ job, long long n_rays, co
       }
       ++k;
     }
-    if (!advance(G, g, cur, a, t, dx, dy, dz, moved, P)) break;
+    if (!cross_face(G, g, cur, g.idx, E, t, true, dx, dy, dz, moved, P)) break;
   }
   counts[r] = k;
 }
@@ -1810,7 +1820,7 @@ static cudaError_t launch_mode(const JobDev* jobs, const ItemDev* items, int n_i
   cudaError_t e = path_smem(k, MaxThreads<R, MODE>::value, cfg.anc, &dyn);
   if (e != cudaSuccess) return e;
   k<<<MODE == 2 ? cfg.blocks_tiled : cfg.blocks, block, dyn, s>>>(jobs, items, n_items, counter, total, cfg.refill,
-                                                                  q, T, cfg.anc);
+                                                                  MODE == 2 ? 16 : cfg.ev_batch, q, T, cfg.anc);
   return cudaGetLastError();
 }
 
@@ -2188,11 +2198,10 @@ __global__ void peel_table_kernel(const JobDev* __restrict__ job, PeelTabSpec S,
         continue;
       }
       settle_leaf(g, cur, wd, r64);
-      int ax;
-      const double t = exit_dist(g, k[0], k[1], k[2], ix, iy, iz, ax);
-      if (ax < 0) break;
-      col += g.rho * Num<double>::pow2m(g.lev) * t;
-      if (!advance(G, g, cur, ax, t, k[0], k[1], k[2])) break;
+      const Exit<double> E = exit_face(g, k[0], k[1], k[2], ix, iy, iz);
+      if (!Num<double>::finite(E.t)) break;
+      col += Num<double>::down(g.rho, g.lev) * E.t;
+      if (!cross_face(G, g, cur, g.idx, E, k[0], k[1], k[2])) break;
     }
   }
   out[i] = col;
