@@ -84,7 +84,9 @@ int rt_ctx_set_peel_queue(rt_ctx* ctx, int64_t max_records);
  * next round.  Results are those of the untiled tracer (the same package
  * histories; only the order of the FP64 additions differs).  tile_edge < 0:
  * automatic (tiles whose node words plus one bin's accumulators take at most
- * 48 MB, only when the whole grid's take more); 0: off.  Uses two record
+ * 48 MB, only when the whole grid's take more and, in FP32, when the cells in
+ * frequent use, 12 B x sum over levels of cells x 4^-level, exceed 120 MB and
+ * each bin has at least a package for every 48 of them); 0: off.  Uses two record
  * buffers of up to 2^26 (FP32, 80 B each) or 2^25 (FP64, 144 B each)
  * records.  Returns RT_ERR_INVALID if tile_edge is not a power of two. */
 int rt_ctx_set_tiles(rt_ctx* ctx, int tile_edge);

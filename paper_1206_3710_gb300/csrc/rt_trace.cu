@@ -583,6 +583,20 @@ struct MaxThreads {
   static constexpr int value = (sizeof(R) == 4 && MODE == 2) ? RT_FP32_TILED_BLOCK : 256;
 };
 
+// Whether a lane that meets a refined node goes down to its leaf within the
+// pass, and takes its segment with the others, or one level per pass.  The
+// first keeps more lanes at the segment, but the warp waits for the deepest
+// descent: it pays where descents are frequent (the grids with a stored
+// path) and short.  Tracer and marches, one level against down to the leaf:
+// deep cloud (3 levels) 6.26 / 5.86 ms, discs of 6 and 8 levels 4.77 / 4.62 and
+// 12.2 / 11.8 ms, but of 10 levels (9.2e6 cells) 14.6 / 15.2 ms; FP64, which
+// waits for its pipe anyway, 3.37 / 2.70 ms.  Without a stored path (128^3
+// cloud) 5.23 / 5.63 ms.
+template <typename R, bool PATH>
+__device__ __forceinline__ bool descend_to_leaf(int n_anc) {
+  return PATH && (sizeof(R) == 8 || n_anc <= 8);
+}
+
 // PATH: lanes keep the path above their leaf (n_anc levels) and start the
 // search for a neighbour outside their octet at the deepest stored ancestor
 // it shares, else at the root cell
@@ -1105,6 +1119,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
         }
       }
     };
+    const bool to_leaf = descend_to_leaf<R, PATH>(n_anc);
     // The tracing-only pass.  On large grids it is bound by the SM's random
     // accesses: one 4-byte load and one FP64 reduction per crossing to cells
     // in the L2 run at 1.2e11 per second at most (a kernel that does nothing
@@ -1124,14 +1139,16 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
       if (ev != EV_NONE) return;
       if ((w & RT_INTERIOR) || cur.k < g.lev || ncross >= step_limit) {
         if (w & RT_INTERIOR) {
-          descend_step(g, cur, w, dx, dy, dz, P);
-          if (RT_COUNT_DESCENTS) atomicAdd(&g_descents[0], 1ull);
-          fetch_node();
-          return;
+          do {
+            descend_step(g, cur, w, dx, dy, dz, P);
+            if (RT_COUNT_DESCENTS) atomicAdd(&g_descents[0], 1ull);
+            fetch_node();
+          } while (to_leaf && (w & RT_INTERIOR));
+          if (!to_leaf) return;
         }
         if (cur.k < g.lev) settle_leaf(g, cur, w, r64);
         if (ncross >= step_limit) ev = EV_KILL;
-        return;
+        if (!to_leaf || ev != EV_NONE) return;
       }
       const uint32_t leaf = cur.pending;
       const int lev = g.lev;
@@ -1588,6 +1605,7 @@ __global__ void __launch_bounds__(256, PeelMinBlocks<R, PATH>::value) peel_kerne
 
     // ----------------------------------------------------------------- march
     int ev = st == P_LIVE ? EV_NONE : EV_IDLE;
+    const bool to_leaf = descend_to_leaf<R, PATH>(n_anc);
     // one pass per lane and iteration.  AX >= 0: every live lane of the warp
     // marches along axis AX in direction PL (an axis observer; the work items
     // are observer-major, so this is the common case) and the axis and the
@@ -1613,8 +1631,17 @@ __global__ void __launch_bounds__(256, PeelMinBlocks<R, PATH>::value) peel_kerne
       }
       do {
         if (ev == EV_NONE) {
-          const uint32_t w = ld_node(G.node + cur.pending);
-          const double r64 = Num<R>::load_rho64(G.rho64, cur.pending);
+          uint32_t w = ld_node(G.node + cur.pending);
+          double r64 = Num<R>::load_rho64(G.rho64, cur.pending);
+          while (to_leaf && (w & RT_INTERIOR)) {
+            if (AX >= 0)
+              descend_step(g, cur, w, AX == 0 ? KA : R(0), AX == 1 ? KA : R(0), AX == 2 ? KA : R(0), P);
+            else
+              descend_step(g, cur, w, dx, dy, dz, P);
+            if (RT_COUNT_DESCENTS) atomicAdd(&g_descents[1], 1ull);
+            w = ld_node(G.node + cur.pending);
+            r64 = Num<R>::load_rho64(G.rho64, cur.pending);
+          }
           if (w & RT_INTERIOR) {
             if (AX >= 0)
               descend_step(g, cur, w, AX == 0 ? KA : R(0), AX == 1 ? KA : R(0), AX == 2 ? KA : R(0), P);

@@ -712,6 +712,62 @@ def test_dust_temperature_parity_ranges(rt, ctx, orc, n_lambda, T_min, T_max):
     np.testing.assert_allclose(To[inside], T_true[inside], rtol=1e-9)
 
 
+def _deep_model(depth, seed):
+    """A 2^3 root refined `depth` levels around one corner: most cells lie
+    below level 1, so launches keep the path above the leaf."""
+    L = 8e16
+    rng = np.random.default_rng(seed)
+    desc = synth.grow_tree((2, 2, 2), (L,) * 3, depth,
+                           lambda l, x, y, z: 1e-20 * 10.0 ** rng.uniform(-1, 1, x.size),
+                           lambda l, x, y, z, r: (x < 2) & (y < 2) & (z < 2))
+    optics = synth.Optics(lambda_um=np.array([0.5, 2.0]), kappa_ext=np.array([3e3, 5e2]), albedo=np.array([0.6, 0.4]),
+                          g_hg=np.array([0.4, 0.0]), dnu=np.array([1e13, 1e13]))
+    return desc, optics, [synth.Source("external", bin_energy=np.array([1.0, 2.0]))]
+
+
+@pytest.mark.parametrize("depth", [2, 3, 8])
+def test_descent_in_one_pass_equals_level_by_level(rt, ctx, depth):
+    """Grids of at most 8 levels descend to the leaf within a pass, deeper ones
+    a level per pass; in a batch the deepest grid decides.  A model traced
+    alone and beside a 9-level one has the same package histories (FP32), and
+    the same images up to the order of the FP64 additions."""
+    npk = 4000
+    obs = synth.Observers(dirs=np.array([[0.36, 0.48, 0.8], [0.0, 0.0, -1.0]]), ups=np.array([[0.0, 1.0, 0.0]] * 2),
+                          nx=24, ny=20, fov=(1e17, 1e17))
+    res = []
+    for beside in (False, True):
+        jobs = []
+        for k, d in enumerate((depth, 9)[:1 + beside]):
+            desc, optics, src = _deep_model(d, d)
+            g = rt.Grid(ctx, desc)
+            jobs.append(rt.Job(g, src, optics, absorbed=_zeros(2, g.n_cells), observers=obs,
+                               images=_zeros(2, 2, obs.ny, obs.nx), seed=5, job=k, packets_per_bin=npk,
+                               packet_log=_zeros(2 * npk, 10)))
+        led = rt.rt_trace_batch(ctx, jobs)[0]
+        res.append((jobs[0].params["packet_log"].cpu().numpy(), jobs[0].absorbed.cpu().numpy(),
+                    jobs[0].images.cpu().numpy(), led))
+    (l0, a0, i0, led0), (l1, a1, i1, led1) = res
+    assert led0["n_scatter"] > 500 and led0["n_peel_cross"] > 1000
+    np.testing.assert_array_equal(l0, l1)
+    for k in ("n_cross", "n_scatter", "n_peel_cross", "n_peel_out"):
+        assert led0[k] == led1[k], k
+    np.testing.assert_allclose(a1, a0, rtol=1e-12, atol=1e-14 * a0.max())
+    np.testing.assert_allclose(i1, i0, rtol=1e-12, atol=1e-14 * i0.max())
+
+
+def test_peel_without_scattering(rt, ctx):
+    """A queue that stays empty is sorted and marched with its length on the
+    device only."""
+    desc, optics, src = _deep_model(3, 1)
+    optics.albedo = np.zeros(2)
+    g = rt.Grid(ctx, desc)
+    obs = synth.axis_observers(16, 8e16, "all6")
+    im = _zeros(6, 2, 16, 16)
+    led = rt.rt_peel(ctx, g, src, optics, obs, im, _zeros(2, g.n_cells), seed=2, packets_per_bin=1000)
+    assert led["n_scatter"] == 0 and led["n_peel_cross"] == 0 and not im.any()
+    assert led["absorbed"] + led["escaped"] == pytest.approx(led["emitted"], rel=1e-5)
+
+
 @pytest.mark.parametrize("n", [1, 255, 1023, 1024, 1025, 2049])
 def test_dust_packages_at_chunk_edges(rt, ctx, orc, n):
     """Packages per cell, floor(E / w + u), at the edges of the chunks the
