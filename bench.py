@@ -59,10 +59,10 @@ BYTES_PEEL_CROSS_PACKED = 4
 BYTES_DESCENT = 4
 DESCENTS_TRACE_DEFAULT = 3004187455
 DESCENTS_PEEL_DEFAULT = 5202007659
-# (captured before the present stepping and marching loops: 11.329e9 B /
-# 2.704457093e9 and 1.206e9 B / 1.808753762e9)
-NCU_TRACE_BYTES_PER_CROSSING = None
-NCU_PEEL_BYTES_PER_CROSSING = None
+# (The capture precedes the present stepping and marching loops, which make the
+# same loads, reductions and record moves per crossing.)
+NCU_TRACE_BYTES_PER_CROSSING = 11.329e9 / 2.704457093e9
+NCU_PEEL_BYTES_PER_CROSSING = 1.206e9 / 1.808753762e9
 
 
 def parse():

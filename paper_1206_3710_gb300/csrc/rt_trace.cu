@@ -592,16 +592,19 @@ struct MaxThreads {
 // 12.2 / 11.8 ms, but of 10 levels (9.2e6 cells) 14.6 / 15.2 ms; FP64, which
 // waits for its pipe anyway, 3.37 / 2.70 ms.  Without a stored path (128^3
 // cloud) 5.23 / 5.63 ms.
-template <typename R, bool PATH>
-__device__ __forceinline__ bool descend_to_leaf(int n_anc) {
-  return PATH && (sizeof(R) == 8 || n_anc <= 8);
+// A kernel of its own for each (PATH): deciding it at run time cost the
+// 9.2e6-cell disc 6 %.
+enum { PATH_NONE = 0, PATH_LEVEL = 1, PATH_LEAF = 2 };
+template <typename R>
+static int path_form(int anc) {
+  return anc <= 0 ? PATH_NONE : (sizeof(R) == 8 || anc <= 8 ? PATH_LEAF : PATH_LEVEL);
 }
 
-// PATH: lanes keep the path above their leaf (n_anc levels) and start the
+// PATH (PATH_NONE: no): lanes keep the path above their leaf (n_anc levels) and start the
 // search for a neighbour outside their octet at the deepest stored ancestor
 // it shares, else at the root cell
 template <typename R, bool PEEL, int EST, bool HITS, int MODE, bool LEVELS = false, bool SPLIT = false,
-          bool PATH = false>
+          int PATH = 0>
 __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>::value) trace_kernel(const JobDev* __restrict__ jobs,
                                                                          const ItemDev* __restrict__ items,
                                                                          int n_items,
@@ -1119,7 +1122,7 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
         }
       }
     };
-    const bool to_leaf = descend_to_leaf<R, PATH>(n_anc);
+    constexpr bool to_leaf = PATH == PATH_LEAF;
     // The tracing-only pass.  On large grids it is bound by the SM's random
     // accesses: one 4-byte load and one FP64 reduction per crossing to cells
     // in the L2 run at 1.2e11 per second at most (a kernel that does nothing
@@ -1475,12 +1478,12 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
 #ifndef RT_PEEL_OBS_MAJOR
 #define RT_PEEL_OBS_MAJOR 1
 #endif
-template <typename R, bool PATH>
+template <typename R, int PATH>
 struct PeelMinBlocks {
   static constexpr int value = sizeof(R) == 4 ? RT_PEEL_MIN_BLOCKS - (PATH ? 1 : 0) : 2;
 };
 
-template <typename R, bool TAB, bool PATH = false>
+template <typename R, bool TAB, int PATH = 0>
 __global__ void __launch_bounds__(256, PeelMinBlocks<R, PATH>::value) peel_kernel(const JobDev* __restrict__ jobs,
                                                                            PeelQueue Q,
                                                                            unsigned long long* __restrict__ work,
@@ -1605,7 +1608,7 @@ __global__ void __launch_bounds__(256, PeelMinBlocks<R, PATH>::value) peel_kerne
 
     // ----------------------------------------------------------------- march
     int ev = st == P_LIVE ? EV_NONE : EV_IDLE;
-    const bool to_leaf = descend_to_leaf<R, PATH>(n_anc);
+    constexpr bool to_leaf = PATH == PATH_LEAF;
     // one pass per lane and iteration.  AX >= 0: every live lane of the warp
     // marches along axis AX in direction PL (an axis observer; the work items
     // are observer-major, so this is the common case) and the axis and the
@@ -1840,8 +1843,14 @@ template <typename R, bool PEEL, int EST, bool HITS, int MODE, bool LEVELS, bool
 static cudaError_t launch_mode(const JobDev* jobs, const ItemDev* items, int n_items, unsigned long long* counter,
                                long long total, const LaunchCfg& cfg, const PeelQueue& q, cudaStream_t s,
                                const TileRun& T) {
-  auto k = cfg.anc > 0 ? trace_kernel<R, PEEL, EST, HITS, MODE, LEVELS, SPLIT, true>
-                       : trace_kernel<R, PEEL, EST, HITS, MODE, LEVELS, SPLIT, false>;
+  // the form that descends to the leaf exists for the untiled tracers of the
+  // continuous estimator, in FP64 in place of the level-by-level one
+  constexpr bool leaf_ok = MODE == 0 && EST == RT_EST_CONTINUOUS && !SPLIT;
+  constexpr int deep = leaf_ok && sizeof(R) == 8 ? PATH_LEAF : PATH_LEVEL;
+  const int form = path_form<R>(cfg.anc);
+  auto k = form == PATH_NONE   ? trace_kernel<R, PEEL, EST, HITS, MODE, LEVELS, SPLIT, PATH_NONE>
+           : form == PATH_LEAF ? trace_kernel<R, PEEL, EST, HITS, MODE, LEVELS, SPLIT, leaf_ok ? PATH_LEAF : PATH_LEVEL>
+                               : trace_kernel<R, PEEL, EST, HITS, MODE, LEVELS, SPLIT, deep>;
   const int block = std::min(cfg.block, MaxThreads<R, MODE>::value);
   size_t dyn = 0;
   cudaError_t e = path_smem(k, MaxThreads<R, MODE>::value, cfg.anc, &dyn);
@@ -2150,7 +2159,10 @@ static cudaError_t launch_peel_t(const JobDev* jobs, const PeelQueue& q, unsigne
   int dev = 0, sms = 0, occ = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  auto k = anc > 0 ? peel_kernel<R, TAB, true> : peel_kernel<R, TAB, false>;
+  const int form = path_form<R>(anc);
+  auto k = form == PATH_NONE   ? peel_kernel<R, TAB, PATH_NONE>
+           : form == PATH_LEAF ? peel_kernel<R, TAB, PATH_LEAF>
+                               : peel_kernel<R, TAB, sizeof(R) == 8 ? PATH_LEAF : PATH_LEVEL>;
   size_t dyn = 0;
   cudaError_t e = path_smem(k, 256, anc, &dyn);
   if (e != cudaSuccess) return e;
@@ -2246,14 +2258,14 @@ template <typename R, bool PEEL>
 static cudaError_t occ_t(int block, int* n, int mode, int anc) {
   size_t dyn = 0;
   if (mode == 2) {
-    auto k = anc > 0 ? trace_kernel<R, PEEL, RT_EST_CONTINUOUS, false, 2, false, false, true>
-                     : trace_kernel<R, PEEL, RT_EST_CONTINUOUS, false, 2, false, false, false>;
+    auto k = anc > 0 ? trace_kernel<R, PEEL, RT_EST_CONTINUOUS, false, 2, false, false, PATH_LEVEL>
+                     : trace_kernel<R, PEEL, RT_EST_CONTINUOUS, false, 2, false, false, PATH_NONE>;
     const int b = std::min(block, MaxThreads<R, 2>::value);
     cudaError_t e = path_smem(k, MaxThreads<R, 2>::value, anc, &dyn);
     return e != cudaSuccess ? e : cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k, b, dyn);
   }
-  auto k = anc > 0 ? trace_kernel<R, PEEL, RT_EST_CONTINUOUS, false, 0, false, false, true>
-                   : trace_kernel<R, PEEL, RT_EST_CONTINUOUS, false, 0, false, false, false>;
+  auto k = anc > 0 ? trace_kernel<R, PEEL, RT_EST_CONTINUOUS, false, 0, false, false, PATH_LEAF>
+                   : trace_kernel<R, PEEL, RT_EST_CONTINUOUS, false, 0, false, false, PATH_NONE>;
   cudaError_t e = path_smem(k, MaxThreads<R, 0>::value, anc, &dyn);
   return e != cudaSuccess ? e : cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k, block, dyn);
 }
