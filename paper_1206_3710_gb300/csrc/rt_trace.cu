@@ -306,7 +306,10 @@ __device__ __forceinline__ unsigned long long claim_slot(unsigned long long* ctr
 // does not ask again.  The counter is one address, its atomics take their
 // turns a few ns apart: by the counter alone a launch of 1e5 packages makes
 // 1.2e4 of them, most for nothing.  state (the warp's, in shared memory): 0
-// nothing taken yet, 1 the end was seen, 2 the warp's own taken.
+// nothing taken yet, 1 the end was seen, 2 the warp's own taken.  Lane 0
+// stores it; a __syncwarp on either side of the store orders it against this
+// and the next call's reads (shuffles and ballots bring the lanes together
+// but order no memory).
 __device__ __forceinline__ long long next_work(unsigned long long* counter, long long n, unsigned dead, int leader,
                                                int lane, int& state) {
   const int rank = __popc(dead & ((1u << lane) - 1u));
@@ -315,6 +318,7 @@ __device__ __forceinline__ long long next_work(unsigned long long* counter, long
   if (st == 0) {
     // (every lane is dead at a warp's first refill)
     if (lane == 0) state = 2;
+    __syncwarp();
     return ((long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + rank;
   }
   if (st == 1) return n + rank;
@@ -322,6 +326,7 @@ __device__ __forceinline__ long long next_work(unsigned long long* counter, long
   if (lane == leader) base = atomicAdd(counter, (unsigned long long)__popc(dead));
   base = __shfl_sync(0xFFFFFFFFu, base, leader) + 32ull * gridDim.x * (blockDim.x >> 5);
   if (lane == 0 && (long long)base + __popc(dead) >= n) state = 1;
+  __syncwarp();
   return (long long)base + rank;
 }
 

@@ -1,0 +1,92 @@
+"""Device functions of the tracers and dust kernels on the CPU: their source
+is taken from the .cu / .cuh files as it stands, compiled with g++ over
+cuda_on_host.h (lanes of a warp as threads) and run."""
+import os
+import re
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_1206_3710_gb300", "csrc")
+
+
+def _source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return f.read()
+
+
+def _take(name, start):
+    """The definition that begins at the regular expression `start`, up to its
+    closing brace (and the semicolon of a struct)."""
+    text = _source(name)
+    m = re.search(start, text, re.M)
+    assert m, f"{name}: {start}"
+    i = text.index("{", m.end() - 1 if text[m.end() - 1] == "{" else m.end())
+    depth, j = 0, i
+    while True:
+        depth += {"{": 1, "}": -1}.get(text[j], 0)
+        j += 1
+        if depth == 0:
+            break
+    return text[m.start():j] + (";" if text[j:j + 1] == ";" else "") + "\n"
+
+
+def _run(tmp_path, body, *args):
+    src, exe = tmp_path / "t.cpp", tmp_path / "t"
+    src.write_text('#include "cuda_on_host.h"\n' + body)
+    r = subprocess.run(["g++", "-std=c++17", "-O1", "-pthread", "-ffp-contract=off", "-w", "-I" + HERE, "-I" + CSRC,
+                        str(src), "-o", str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-4000:]
+    r = subprocess.run([str(exe), *map(str, args)], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, (r.returncode, r.stdout[-2000:], r.stderr[-2000:])
+    return r.stdout
+
+
+@pytest.mark.parametrize("n", [0, 1, 31, 33, 128, 129, 1000])
+def test_work_items_are_given_out_once(tmp_path, n):
+    """next_work: the warps of a grid take every item exactly once when a
+    lane's store to the warp's state reaches the other lanes no sooner than
+    the memory model promises it (at a __syncwarp)."""
+    body = _take("rt_trace.cu", r"^__device__ __forceinline__ long long next_work\(") + r"""
+int main(int argc, char** argv) {
+  const long long n = atoll(argv[1]);
+  gridDim.x = 2;
+  blockDim.x = 64;
+  unsigned long long counter = 0;
+  std::vector<std::atomic<int>> given((size_t)n);
+  for (auto& g : given) g = 0;
+  for (unsigned b = 0; b < gridDim.x; ++b)
+    for (unsigned w = 0; w < blockDim.x / 32; ++w) {
+      on_lanes(32, [&](int lane) {
+        threadIdx.x = 32 * w + (unsigned)lane;
+        blockIdx.x = b;
+        int state = 0;  // this lane's view of the warp's shared variable
+        warp_state->view[lane] = &state;
+        unsigned dead = 0xFFFFFFFFu, done = 0u, rnd = 12345u + 7u * b + w;
+        while (done != 0xFFFFFFFFu) {
+          const bool mine = dead >> lane & 1u;
+          const long long i = next_work(&counter, n, dead, __ffs(dead) - 1, lane, state);
+          if (mine && i >= 0 && i < n) given[(size_t)i].fetch_add(1);
+          // lanes without an item are done, some of the others die (all lanes
+          // agree on the masks, as by a ballot)
+          warp_state->slot[lane] = mine && i >= n;
+          meet(0xFFFFFFFFu);
+          for (int l = 0; l < 32; ++l)
+            if (warp_state->slot[l]) done |= 1u << l;
+          rnd = rnd * 1664525u + 1013904223u;
+          dead = (rnd >> 3 | rnd << 7) & ~done;
+          if (dead == 0u) dead = ~done;
+          meet(0xFFFFFFFFu);
+        }
+      });
+    }
+  for (long long i = 0; i < n; ++i)
+    if (given[(size_t)i] != 1) {
+      printf("item %lld given %d times\n", i, given[(size_t)i].load());
+      return 1;
+    }
+  return 0;
+}
+"""
+    _run(tmp_path, body, n)
