@@ -142,7 +142,8 @@ struct Num<double> {
   static __device__ __forceinline__ bool same(double x, double y) { return b(x) == b(y); }
   static __device__ __forceinline__ bool ge(double x, double y) { return b(x) >= b(y); }
   static __device__ __forceinline__ bool pos(double x) { return b(x) != 0ull; }
-  static __device__ __forceinline__ bool finite(double x) { return __double2hiint(x) < 0x7FF00000; }
+  // (the device's NaN has the sign bit: unsigned, so that it ranks above inf here too)
+  static __device__ __forceinline__ bool finite(double x) { return (uint32_t)__double2hiint(x) < 0x7FF00000u; }
   static __device__ __forceinline__ bool not_neg(double d) { return __double2hiint(d) >= 0 || (b(d) << 1) == 0ull; }
   static __device__ __forceinline__ bool above(double f, double h) { return b(f) > b(h); }
   static __device__ __forceinline__ double one_if(uint32_t u) { return __hiloint2double(u ? 0x3FF00000 : 0, 0); }

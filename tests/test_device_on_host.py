@@ -90,3 +90,30 @@ int main(int argc, char** argv) {
 }
 """
     _run(tmp_path, body, n)
+
+
+def _num(kind):
+    """The number traits, without the accessors of the device tables."""
+    t = _take("rt_device.cuh", r"^template <>\nstruct Num<%s> \{" % kind)
+    return "template <typename R>\nstruct Num;\n" + re.sub(r"^.*\b(BinDev|ItemDev|JobDev)\b.*\}\n", "", t, flags=re.M)
+
+
+@pytest.mark.parametrize("kind", ["float", "double"])
+def test_finite_distance(tmp_path, kind):
+    """Num::finite tells an exit distance (not negative) from the infinity and
+    the NaNs, of either sign, that a zero direction component gives."""
+    body = "#include <cmath>\n#include <float.h>\n" + _num(kind) + r"""
+typedef KIND R;
+int main() {
+  const R big = sizeof(R) == 4 ? (R)FLT_MAX : (R)DBL_MAX, tiny = sizeof(R) == 4 ? (R)1e-45f : (R)4.9e-324;
+  const R yes[] = {R(0), tiny, R(0.5), R(1.7320508), big};
+  const R nan = (R)NAN, no[] = {(R)INFINITY, nan, -nan, R(0) * (R)INFINITY};
+  int bad = 0;
+  for (R v : yes)
+    if (!Num<R>::finite(v)) printf("%g is not finite\n", (double)v), bad = 1;
+  for (R v : no)
+    if (Num<R>::finite(v)) printf("%s%g is finite\n", std::signbit(v) ? "-" : "+", (double)fabs(v)), bad = 1;
+  return bad;
+}
+""".replace("KIND", kind)
+    _run(tmp_path, body)
