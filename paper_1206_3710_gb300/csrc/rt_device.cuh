@@ -53,10 +53,10 @@ struct Num<float> {
   static __device__ __forceinline__ void sincos2pi(float u, float* s, float* c) { sincospif(2.0f * u, s, c); }
   static __device__ __forceinline__ float inf() { return CUDART_INF_F; }
   // 1 for d > 0, else 0: the offset of the face ahead.  A saturated multiply,
-  // so that the stepping loop's selects stay off the integer/compare pipe
-  // (a component below 1e-38 has an infinite reciprocal: its face is never
-  // the nearest, whatever comes out here)
-  static __device__ __forceinline__ float ahead(float d) { return __saturatef(d * 3.0e38f); }
+  // so that the stepping loop's selects stay off the integer/compare pipe.
+  // By the largest float: a component for which that gives a fraction (below
+  // 2.94e-39) has an infinite reciprocal, and its face is never the nearest
+  static __device__ __forceinline__ float ahead(float d) { return __saturatef(d * 3.4028234663852886e38f); }
   // offset f moved by t along d, kept in [0, 1]
   static __device__ __forceinline__ float moved01(float f, float t, float d) { return __saturatef(fmaf(t, d, f)); }
   static __device__ __forceinline__ float min_(float a, float b) { return fminf(a, b); }

@@ -117,3 +117,33 @@ int main() {
 }
 """.replace("KIND", kind)
     _run(tmp_path, body)
+
+
+def test_face_ahead_of_tiny_components(tmp_path):
+    """Num<float>::ahead is exactly 0 or 1 for every direction component whose
+    reciprocal is finite: a fraction there would put the face ahead inside the
+    cell, at distance zero for a package that sits on it.  Every float from
+    the smallest to twice the smallest with a finite reciprocal, and its
+    negative, then powers of two up to 1."""
+    body = _num("float") + _take("rt_device.cuh", r"^template <typename R>\n__device__ __forceinline__ R inv_abs\(") + r"""
+int main() {
+  long long bad = 0;
+  auto look = [&](float d) {
+    const float s = Num<float>::ahead(d), i = inv_abs(d);
+    const bool ok = d > 0.0f ? (s == 1.0f || i == INFINITY) && s >= 0.0f && s <= 1.0f : s == 0.0f;
+    if (!ok && bad++ < 3) printf("d = %g (1/d = %g): ahead %.9g\n", d, i, s);
+  };
+  look(0.0f);
+  look(-0.0f);
+  for (unsigned u = 1; u <= 1u << 22; ++u) {
+    look(__uint_as_float(u));
+    look(-__uint_as_float(u));
+  }
+  for (float d = 1.0f; d > 1e-38f; d *= 0.5f) {
+    look(d);
+    look(-d);
+  }
+  return bad != 0;
+}
+"""
+    _run(tmp_path, body)
