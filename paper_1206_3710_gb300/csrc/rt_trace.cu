@@ -1844,18 +1844,24 @@ static cudaError_t path_smem(K kernel, int max_block, int anc, size_t* bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*bytes);
 }
 
+// the tracer for lanes that store anc levels of the path: the form that
+// descends to the leaf exists for the untiled tracers of the continuous
+// estimator, in FP64 in place of the level-by-level one
+template <typename R, bool PEEL, int EST, bool HITS, int MODE, bool LEVELS, bool SPLIT>
+static auto pick_tracer(int anc) {
+  constexpr bool leaf_ok = MODE == 0 && EST == RT_EST_CONTINUOUS && !SPLIT;
+  constexpr int deep = leaf_ok && sizeof(R) == 8 ? PATH_LEAF : PATH_LEVEL;
+  const int form = path_form<R>(anc);
+  return form == PATH_NONE   ? trace_kernel<R, PEEL, EST, HITS, MODE, LEVELS, SPLIT, PATH_NONE>
+         : form == PATH_LEAF ? trace_kernel<R, PEEL, EST, HITS, MODE, LEVELS, SPLIT, leaf_ok ? PATH_LEAF : PATH_LEVEL>
+                             : trace_kernel<R, PEEL, EST, HITS, MODE, LEVELS, SPLIT, deep>;
+}
+
 template <typename R, bool PEEL, int EST, bool HITS, int MODE, bool LEVELS, bool SPLIT>
 static cudaError_t launch_mode(const JobDev* jobs, const ItemDev* items, int n_items, unsigned long long* counter,
                                long long total, const LaunchCfg& cfg, const PeelQueue& q, cudaStream_t s,
                                const TileRun& T) {
-  // the form that descends to the leaf exists for the untiled tracers of the
-  // continuous estimator, in FP64 in place of the level-by-level one
-  constexpr bool leaf_ok = MODE == 0 && EST == RT_EST_CONTINUOUS && !SPLIT;
-  constexpr int deep = leaf_ok && sizeof(R) == 8 ? PATH_LEAF : PATH_LEVEL;
-  const int form = path_form<R>(cfg.anc);
-  auto k = form == PATH_NONE   ? trace_kernel<R, PEEL, EST, HITS, MODE, LEVELS, SPLIT, PATH_NONE>
-           : form == PATH_LEAF ? trace_kernel<R, PEEL, EST, HITS, MODE, LEVELS, SPLIT, leaf_ok ? PATH_LEAF : PATH_LEVEL>
-                               : trace_kernel<R, PEEL, EST, HITS, MODE, LEVELS, SPLIT, deep>;
+  auto k = pick_tracer<R, PEEL, EST, HITS, MODE, LEVELS, SPLIT>(cfg.anc);
   const int block = std::min(cfg.block, MaxThreads<R, MODE>::value);
   size_t dyn = 0;
   cudaError_t e = path_smem(k, MaxThreads<R, MODE>::value, cfg.anc, &dyn);
@@ -2259,28 +2265,27 @@ cudaError_t build_peel_table(const JobDev* job_dev, const PeelTabSpec& spec, dou
   return cudaGetLastError();
 }
 
-template <typename R, bool PEEL>
-static cudaError_t occ_t(int block, int* n, int mode, int anc) {
+// blocks per SM of the plain tracer (MODE 0 or 2) with the same path levels
+template <typename R, bool PEEL, int MODE>
+static cudaError_t occ_t(int block, int* n, int anc) {
+  auto k = pick_tracer<R, PEEL, RT_EST_CONTINUOUS, false, MODE, false, false>(anc);
   size_t dyn = 0;
-  if (mode == 2) {
-    auto k = anc > 0 ? trace_kernel<R, PEEL, RT_EST_CONTINUOUS, false, 2, false, false, PATH_LEVEL>
-                     : trace_kernel<R, PEEL, RT_EST_CONTINUOUS, false, 2, false, false, PATH_NONE>;
-    const int b = std::min(block, MaxThreads<R, 2>::value);
-    cudaError_t e = path_smem(k, MaxThreads<R, 2>::value, anc, &dyn);
-    return e != cudaSuccess ? e : cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k, b, dyn);
-  }
-  auto k = anc > 0 ? trace_kernel<R, PEEL, RT_EST_CONTINUOUS, false, 0, false, false, PATH_LEAF>
-                   : trace_kernel<R, PEEL, RT_EST_CONTINUOUS, false, 0, false, false, PATH_NONE>;
-  cudaError_t e = path_smem(k, MaxThreads<R, 0>::value, anc, &dyn);
-  return e != cudaSuccess ? e : cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k, block, dyn);
+  cudaError_t e = path_smem(k, MaxThreads<R, MODE>::value, anc, &dyn);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k, std::min(block, MaxThreads<R, MODE>::value), dyn);
+}
+
+template <typename R, bool PEEL>
+static cudaError_t occ_mode(int block, int* n, int mode, int anc) {
+  return mode == 2 ? occ_t<R, PEEL, 2>(block, n, anc) : occ_t<R, PEEL, 0>(block, n, anc);
 }
 
 cudaError_t trace_occupancy(int precision, bool peel, int block, int* blocks_per_sm, int mode, int anc) {
   if (precision == 64)
-    return peel ? occ_t<double, true>(block, blocks_per_sm, mode, anc)
-                : occ_t<double, false>(block, blocks_per_sm, mode, anc);
-  return peel ? occ_t<float, true>(block, blocks_per_sm, mode, anc)
-              : occ_t<float, false>(block, blocks_per_sm, mode, anc);
+    return peel ? occ_mode<double, true>(block, blocks_per_sm, mode, anc)
+                : occ_mode<double, false>(block, blocks_per_sm, mode, anc);
+  return peel ? occ_mode<float, true>(block, blocks_per_sm, mode, anc)
+              : occ_mode<float, false>(block, blocks_per_sm, mode, anc);
 }
 
 cudaError_t launch_walk(int precision, const JobDev* job_dev, long long n_rays, const double* origins,

@@ -147,3 +147,70 @@ int main() {
 }
 """
     _run(tmp_path, body)
+
+
+def test_occupancy_is_the_launched_tracers(tmp_path):
+    """A launch's grid is sized by the occupancy of the tracer that it starts:
+    for both precisions, with and without peel-off, untiled and tiled, and
+    every number of stored path levels, the kernel, block size and dynamic
+    shared memory that the occupancy is asked for are the launch's."""
+    text = _source("rt_trace.cu")
+    form = re.search(r"^enum \{ PATH_NONE.*?^\}\n", text, re.M | re.S).group(0)
+    host = text[text.index("template <typename K>\nstatic cudaError_t path_smem("):]
+    host = host[:host.index("template <typename R, bool PEEL, int EST, bool HITS, bool LEVELS = false>\nstatic")]
+    occ = text[text.rindex("template <", 0, text.index("static cudaError_t occ_t(")):]
+    occ = occ[:occ.index("cudaError_t launch_walk(")]
+    code = re.sub(r"(\w+)<<<(.*?)>>>\(", r"launch_of(\1, \2)(", form + host + occ, flags=re.S)
+    depth = int(re.search(r"#define RT_ANC_MAX (\d+)", _source("rt_internal.cuh")).group(1))
+    body = r"""
+enum cudaError_t { cudaSuccess, cudaErrorOther };
+enum { cudaFuncAttributeMaxDynamicSharedMemorySize };
+typedef void* cudaStream_t;
+enum { RT_EST_CONTINUOUS = 0, RT_EST_ANALOG = 1 };
+struct JobDev; struct ItemDev;
+struct PeelQueue {}; struct TileRun {};
+struct LaunchCfg { int block = 256, blocks = 1, refill = 8, blocks_tiled = 1, ev_batch = 12, anc = 0; };
+struct Use { const void* k = nullptr; int block = 0; size_t dyn = 0; };
+static Use launched, asked;
+template <typename R, int MODE> struct MaxThreads { static constexpr int value = sizeof(R) == 4 && MODE == 2 ? 224 : 256; };
+template <typename R, bool PEEL, int EST, bool HITS, int MODE, bool LEVELS = false, bool SPLIT = false, int PATH = 0>
+void trace_kernel() { static volatile int one; one = PATH; }
+template <typename K> cudaError_t cudaFuncSetAttribute(K, int, int) { return cudaSuccess; }
+static cudaError_t cudaGetLastError() { return cudaSuccess; }
+template <typename K> cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int* n, K k, int block, size_t dyn) {
+  asked.k = (const void*)k; asked.block = block; asked.dyn = dyn; *n = 1;
+  return cudaSuccess;
+}
+template <typename K> auto launch_of(K k, int, int block, size_t dyn, cudaStream_t) {
+  launched.k = (const void*)k; launched.block = block; launched.dyn = dyn;
+  return [](auto&&...) {};
+}
+""" + code + r"""
+template <typename R, bool PEEL, int MODE>
+static int look(int block, int anc) {
+  LaunchCfg cfg;
+  cfg.block = block;
+  cfg.anc = anc;
+  int n = 0;
+  launch_mode<R, PEEL, RT_EST_CONTINUOUS, false, MODE, false, false>(nullptr, nullptr, 0, nullptr, 0, cfg, PeelQueue(),
+                                                                    nullptr, TileRun());
+  trace_occupancy(8 * sizeof(R), PEEL, block, &n, MODE, anc);
+  if (launched.k == asked.k && launched.block == asked.block && launched.dyn == asked.dyn) return 0;
+  printf("FP%d peel %d mode %d block %d levels %d: kernel %s, block %d / %d, shared %zu / %zu\n", (int)(8 * sizeof(R)),
+         PEEL, MODE, block, anc, launched.k == asked.k ? "same" : "another", launched.block, asked.block, launched.dyn,
+         asked.dyn);
+  return 1;
+}
+int main() {
+  int bad = 0;
+  for (int block : {32, 256})
+    for (int anc = 0; anc <= DEPTH; ++anc) {
+      bad += look<float, false, 0>(block, anc) + look<float, true, 0>(block, anc);
+      bad += look<float, false, 2>(block, anc) + look<float, true, 2>(block, anc);
+      bad += look<double, false, 0>(block, anc) + look<double, true, 0>(block, anc);
+      bad += look<double, false, 2>(block, anc) + look<double, true, 2>(block, anc);
+    }
+  return bad != 0;
+}
+""".replace("DEPTH", str(depth))
+    _run(tmp_path, body)
