@@ -735,8 +735,9 @@ __device__ __forceinline__ double weighted_emission(const EmitBin* bins, const u
 // plain solve's T; T_min / T_max where the target lies outside (looked at
 // when a step first runs into that end).  Eight lanes share a cell's bins:
 // with a thread per cell the 27,200 cells of a small disc with 12 bins took
-// 1.58 ms, most of it latency of 213 blocks, now 0.15 ms.  Newton stops once a step is
-// below 1e-9 T: it converges quadratically, what is left is below 1e-16.
+// 1.58 ms, most of it latency of 213 blocks, now 0.15 ms.  Newton stops once a
+// step is below 1e-10 T: a step of d T leaves about x / 2 d^2, x = h nu / k T of
+// the bins that emit (below 710, where a term is zero): below 4e-18.
 __global__ void __launch_bounds__(128) temperature_weighted_kernel(
     const double* __restrict__ rhs, const double* __restrict__ w, const uint8_t* __restrict__ use, long long n,
     const uint32_t* __restrict__ child, const double* __restrict__ rho64, const uint8_t* __restrict__ level, double h0,
@@ -786,7 +787,7 @@ __global__ void __launch_bounds__(128) temperature_weighted_kernel(
         }
         const double step = fabs(tn - t);
         t = tn;
-        if (step <= 1e-9 * t || (hi - lo) <= 1e-14 * lo) break;
+        if (step <= 1e-10 * t || (hi - lo) <= 1e-14 * lo) break;
       }
       out = t;
     }

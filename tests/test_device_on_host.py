@@ -214,3 +214,118 @@ int main() {
 }
 """.replace("DEPTH", str(depth))
     _run(tmp_path, body)
+
+
+def test_ali_temperatures(tmp_path):
+    """temperature_weighted_kernel against bisection in long double, 40 cells:
+    each cell's T within 1e-13 of the root of sum_b w_b E_b(T) = rhs / (rho V)
+    whatever its start (rounding of the sum and of x = h nu / k T, eps each,
+    moves T by a few eps; 1e-13 leaves room for weights near 1e-3), T_min and
+    T_max where the target lies outside, zero density and cells not in use
+    left out.  Then, where Newton's factor is largest (one bin, x near 690),
+    500 cells that start just under 1e-9 from the root: their mean error is
+    below 1e-16.  A step of 0.99e-9 that ends the iteration leaves x / 2 times
+    its square, 3.4e-16, on the same side in every cell; rounding (2 eps of
+    either sign) averages to 2e-17."""
+    names = [r"^struct EmitBin \{", r"^__device__ __forceinline__ void planck_and_deriv\(",
+             r"^__device__ __forceinline__ double leaf_mass\(", r"^__device__ __forceinline__ void emit_setup\(",
+             r"^__device__ __forceinline__ double emit_term\(", r"^__device__ __forceinline__ double weighted_emission\("]
+    consts = "".join(re.findall(r"^#define (?:\w+_CGS|FOUR_PI) .*\n", _source("rt_dust.cu"), re.M))
+    body = r"""
+#include "rt_planck.cuh"
+static inline void __syncthreads() { meet(0xFFu); }
+namespace rtk {
+alignas(16) unsigned char smem[1 << 15];
+""" + consts + "".join(_take("rt_dust.cu", n) for n in names) + \
+        _take("rt_dust.cu", r"^__global__ void __launch_bounds__\(128\) temperature_weighted_kernel\(") + r"""
+}
+using namespace rtk;
+typedef long double LD;
+static LD emission(const std::vector<double>& lam, const std::vector<double>& kabs, const std::vector<double>& dnu,
+                   const double* w, long long n, long long c, LD T) {
+  LD s = 0;
+  for (size_t b = 0; b < lam.size(); ++b) {
+    // (the bin's frequency and h nu are rounded once, for all cells)
+    const double nud = C_CGS / (lam[b] * 1e-4), hnu = H_CGS * nud;
+    const LD nu = nud;
+    s += (LD)w[b * n + c] * 4 * (LD)M_PIl * (LD)kabs[b] * (LD)dnu[b] * 2 * (LD)H_CGS * nu * nu * nu /
+         ((LD)C_CGS * (LD)C_CGS) / expm1l((LD)hnu / ((LD)K_CGS * T));
+  }
+  return s;
+}
+static std::vector<double> solve(const std::vector<double>& lam, const std::vector<double>& kabs,
+                                 const std::vector<double>& dnu, const std::vector<double>& w,
+                                 const std::vector<double>& rhs, const std::vector<double>& rho,
+                                 const std::vector<uint8_t>& use, std::vector<double> T, double Tmin, double Tmax) {
+  const long long n = (long long)rhs.size();
+  std::vector<uint32_t> child(n, 0u);
+  std::vector<uint8_t> level(n, 1);
+  gridDim.x = 1;
+  blockDim.x = 8;
+  on_lanes(8, [&](int) {
+    temperature_weighted_kernel(rhs.data(), w.data(), use.data(), n, child.data(), rho.data(), level.data(), 2.0,
+                                lam.data(), kabs.data(), dnu.data(), (int)lam.size(), Tmin, Tmax, T.data());
+  });
+  return T;
+}
+int main() {
+  int bad = 0;
+  unsigned rnd = 1u;
+  auto uni = [&] { return (rnd = rnd * 1664525u + 1013904223u) * 2.3283064365386963e-10; };
+  {
+    const int nl = 12;
+    const long long n = 40;
+    std::vector<double> lam, kabs, dnu, w(nl * n), rhs(n), rho(n), T0(n), Tt(n);
+    for (int b = 0; b < nl; ++b) {
+      lam.push_back(0.3 * pow(10.0, 0.35 * b));
+      kabs.push_back(300.0 * pow(lam[b] / 0.55, -1.8));
+      dnu.push_back(0.8 * C_CGS / (lam[b] * 1e-4));
+    }
+    std::vector<uint8_t> use(n, 1);
+    for (long long c = 0; c < n; ++c) {
+      for (int b = 0; b < nl; ++b) w[b * n + c] = 1.0 - 0.999 * uni();
+      rho[c] = 1e-19 * (1 + uni());  // V = 1 at level 1 of h0 = 2
+      Tt[c] = 4.0 * pow(500.0, uni());
+      if (c == 0) Tt[c] = 2.0;     // below T_min
+      if (c == 1) Tt[c] = 5000.0;  // above T_max
+      rhs[c] = (double)((LD)rho[c] * emission(lam, kabs, dnu, w.data(), n, c, Tt[c]));
+      T0[c] = c % 4 == 0 ? 0.0 : c % 4 == 1 ? 2.7 : c % 4 == 2 ? 3000.0 : Tt[c] * 1.3;
+    }
+    rho[2] = 0.0;
+    use[3] = 0;
+    const std::vector<double> T = solve(lam, kabs, dnu, w, rhs, rho, use, T0, 2.7, 3000.0);
+    for (long long c = 0; c < n; ++c) {
+      LD lo = 2.7L, hi = 3000.0L;
+      const LD target = c == 2 ? 0 : (LD)rhs[c] / (LD)rho[c];
+      if (c != 2)
+        while (hi - lo > 1e-17L * lo) {
+          const LD mid = (lo + hi) / 2;
+          if (mid == lo || mid == hi) break;
+          (emission(lam, kabs, dnu, w.data(), n, c, mid) < target ? lo : hi) = mid;
+        }
+      const LD want = c == 0 || c == 2 ? 2.7L : c == 1 ? 3000.0L : c == 3 ? (LD)T0[3] : lo;
+      if (fabsl((LD)T[c] - want) > 1e-13L * want) {
+        printf("cell %lld: T %.17g, not %.17Lg\n", c, T[c], want);
+        bad = 1;
+      }
+    }
+  }
+  {
+    const long long n = 500;
+    const std::vector<double> lam{1.0}, kabs{100.0}, dnu{1e14};
+    std::vector<double> w(n, 1.0), rhs(n), rho(n, 1.0), T0(n), Tt(n);
+    for (long long c = 0; c < n; ++c) {
+      Tt[c] = H_CGS * C_CGS / 1e-4 / (K_CGS * (680.0 + 20.0 * uni()));
+      rhs[c] = (double)emission(lam, kabs, dnu, w.data(), n, c, (LD)Tt[c]);
+      T0[c] = Tt[c] * (1.0 + (c & 1 ? 0.99e-9 : -0.99e-9));
+    }
+    const std::vector<double> T = solve(lam, kabs, dnu, w, rhs, rho, std::vector<uint8_t>(n, 1), T0, 2.7, 3000.0);
+    LD mean = 0;
+    for (long long c = 0; c < n; ++c) mean += ((LD)T[c] - (LD)Tt[c]) / (LD)Tt[c] / n;
+    printf("mean error %.3Lg\n", mean);
+    if (fabsl(mean) > 1e-16L) bad = 1;
+  }
+  return bad;
+}
+"""
+    _run(tmp_path, body)
