@@ -15,9 +15,11 @@ workload on the host cores.
 from __future__ import annotations
 
 import argparse
+import hashlib
 import json
 import math
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -48,9 +50,10 @@ BYTES_PEEL_CROSS_PACKED = 4
 # launch of one step of the same cloud at 128^3 root cells (tiles of 64^3,
 # 1e6 packages per wavelength: 11.33 GB for 2.704e9 trace crossings, 1.206 GB
 # for 1.809e9 peel-off crossings).  The bench line scales them by its own
-# crossings on the default 256^3 workload (None whenever a kernel changes
-# until it is captured again).  The tracer's figure is an upper bound there:
-# the 128^3 case crosses tile faces twice as often per cell crossing.
+# crossings on the default 256^3 workload, and gives none when a kernel has
+# changed since (NCU_KERNEL_DIGEST: kernel_digest() of the captured sources).
+# The tracer's figure is an upper bound there: the 128^3 case crosses tile
+# faces twice as often per cell crossing.
 # node descents per step of the default 256^3 cloud (a global read of an
 # interior cell's child word each: 4 B in the roofline unit), counted with a
 # build compiled with RT_COUNT_DESCENTS=1 (rt_descent_counts; the package
@@ -59,10 +62,26 @@ BYTES_PEEL_CROSS_PACKED = 4
 BYTES_DESCENT = 4
 DESCENTS_TRACE_DEFAULT = 3004187455
 DESCENTS_PEEL_DEFAULT = 5202007659
-# (The capture precedes the present stepping and marching loops, which make the
-# same loads, reductions and record moves per crossing.)
 NCU_TRACE_BYTES_PER_CROSSING = 11.329e9 / 2.704457093e9
 NCU_PEEL_BYTES_PER_CROSSING = 1.206e9 / 1.808753762e9
+NCU_KERNEL_DIGEST = "45a5fffa211a96c2"
+
+
+def kernel_digest():
+    """Digest of the tracer and march sources without comments and white space."""
+    h = hashlib.sha256()
+    for name in ("rt_trace.cu", "rt_device.cuh", "rt_internal.cuh", "philox.cuh"):
+        with open(os.path.join(ROOT, "paper_1206_3710_gb300", "csrc", name)) as f:
+            h.update(re.sub(r"//[^\n]*|/\*.*?\*/|\s+", "", f.read(), flags=re.S).encode())
+    return h.hexdigest()[:16]
+
+
+def captured_traffic(ledger):
+    """DRAM bytes of a step's tracer launches and of its peel-off kernel, from
+    the capture; None when it is of other kernels."""
+    if NCU_KERNEL_DIGEST != kernel_digest():
+        return None, None
+    return (NCU_TRACE_BYTES_PER_CROSSING * ledger["n_cross"], NCU_PEEL_BYTES_PER_CROSSING * ledger["n_peel_cross"])
 
 
 def parse():
@@ -432,11 +451,7 @@ def main():
         peel_bytes += BYTES_DESCENT * DESCENTS_PEEL_DEFAULT
         peel_packed += BYTES_DESCENT * DESCENTS_PEEL_DEFAULT
     achieved = trace_bytes / (kern_ms * 1e-3) / 1e9
-    trace_traffic = peel_traffic = None
-    if default_cloud and NCU_TRACE_BYTES_PER_CROSSING is not None:
-        trace_traffic = NCU_TRACE_BYTES_PER_CROSSING * L0["n_cross"]
-    if default_cloud and NCU_PEEL_BYTES_PER_CROSSING is not None:
-        peel_traffic = NCU_PEEL_BYTES_PER_CROSSING * L0["n_peel_cross"]
+    trace_traffic, peel_traffic = captured_traffic(L0) if default_cloud else (None, None)
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": trace_traffic,
             "traffic_basis": "per step: ncu DRAM bytes per crossing of a 128^3 step, times this step's crossings",
