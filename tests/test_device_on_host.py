@@ -329,3 +329,63 @@ int main() {
 }
 """
     _run(tmp_path, body)
+
+
+@pytest.mark.parametrize("hx,short_form", [(8.6e-4, True), (1.09e-3, True), (1.11e-3, False), (1.7e-3, False)])
+def test_wide_temperature_tables(tmp_path, hx, short_form):
+    """dust_temperature on tables of log E = 5 log T (E = T^5, an exactly
+    linear interpolant) of spacing hx: the short form of the inversion serves
+    every cell inside the table to 1e-14 where its series holds, and is not
+    begun where it does not."""
+    body = r"""
+struct double2 { double x, y; };
+enum cudaError_t { cudaSuccess };
+typedef void* cudaStream_t;
+static cudaError_t cudaGetLastError() { return cudaSuccess; }
+#define __log2f(x) log2f(x)
+static inline void __syncthreads() {}
+#include "rt_planck.cuh"
+namespace rtk {
+alignas(16) float lg[8192];
+static long long quotients, general;
+static double quotient(double a, double b) { ++quotients; return a / b; }
+static double solve_by_table(double A, double mass, const double*, const double*, const double*, int, double, double,
+                             const double*, int) { ++general; return pow(A / mass, 0.2); }
+""" + _take("rt_dust.cu", r"^struct InvNode \{") + \
+        _take("rt_dust.cu", r"^__device__ __forceinline__ double leaf_mass\(") + \
+        _take("rt_dust.cu", r"^__global__ void __launch_bounds__\(256, 4\) temperature_kernel\(") + \
+        re.sub(r"<<<.*?>>>", "", _take("rt_dust.cu", r"^cudaError_t dust_temperature\("), flags=re.S) + r"""
+}
+using namespace rtk;
+int main(int argc, char** argv) {
+  const int nt = 8192, n = 2000;
+  const double hx = atof(argv[1]);
+  std::vector<double> table(12 * nt + 2), rho(n, 1.0), A(n), T(n), want(n);
+  double* tab = (double*)(((uintptr_t)table.data() + 15) / 16 * 16);
+  for (int i = 0; i < nt; ++i) {
+    InvNode N{};
+    N.T = 2.7 * exp(i * hx);
+    N.inv_e = 1.0 / pow(N.T, 5.0);
+    N.c1 = 5.0 * hx;
+    N.hx = hx;
+    ((InvNode*)(tab + 3 * nt))[i] = N;
+    ((float*)(tab + 11 * nt))[i] = (float)(5.0 * log2(N.T));
+  }
+  std::vector<uint32_t> child(n, 0u);
+  std::vector<uint8_t> level(n, 0);
+  for (int c = 0; c < n; ++c) {
+    want[c] = 2.7 * exp(hx * (2.0 + (nt - 6.0) * (c + 0.37) / n));
+    A[c] = pow(want[c], 5.0);
+  }
+  gridDim.x = 1;
+  blockDim.x = 1;
+  dust_temperature(A.data(), 1, n, child.data(), rho.data(), level.data(), 1.0, nullptr, nullptr, nullptr, 1, 2.7,
+                   2.7 * exp((nt - 1) * hx), tab, nt, T.data(), 1, nullptr);
+  double far = 0.0;
+  for (int c = 0; c < n; ++c) far = std::max(far, fabs(T[c] / want[c] - 1.0));
+  printf("%lld quotients, %lld general, error %.2g\n", quotients, general, far);
+  const bool ok = atoi(argv[2]) ? quotients == n && general == 0 : quotients == 0 && general == n;
+  return !(ok && far < 1e-14);
+}
+"""
+    _run(tmp_path, body, hx, int(short_form))
