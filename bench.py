@@ -48,7 +48,7 @@ BYTES_PEEL_CROSS_PACKED = 4
 # the tracer (all its launches in a step: the emission round and the tiled
 # rounds) and of the deferred peel-off kernel, from an ncu capture of every
 # launch of one step of the same cloud at 128^3 root cells (tiles of 64^3,
-# 1e6 packages per wavelength: 11.33 GB for 2.704e9 trace crossings, 1.206 GB
+# 1e6 packages per wavelength: 11.39 GB for 2.704e9 trace crossings, 1.210 GB
 # for 1.809e9 peel-off crossings).  The bench line scales them by its own
 # crossings on the default 256^3 workload, and gives none when a kernel has
 # changed since (NCU_KERNEL_DIGEST: kernel_digest() of the captured sources).
@@ -62,9 +62,9 @@ BYTES_PEEL_CROSS_PACKED = 4
 BYTES_DESCENT = 4
 DESCENTS_TRACE_DEFAULT = 3004187455
 DESCENTS_PEEL_DEFAULT = 5202007659
-NCU_TRACE_BYTES_PER_CROSSING = 11.329e9 / 2.704457093e9
-NCU_PEEL_BYTES_PER_CROSSING = 1.206e9 / 1.808753762e9
-NCU_KERNEL_DIGEST = "45a5fffa211a96c2"
+NCU_TRACE_BYTES_PER_CROSSING = 11.393e9 / 2.704457093e9
+NCU_PEEL_BYTES_PER_CROSSING = 1.210e9 / 1.808753762e9
+NCU_KERNEL_DIGEST = "44cf461bedf688c6"
 
 
 def kernel_digest():
