@@ -65,7 +65,9 @@ typedef struct rt_server rt_server;
 
 /* Create a context on CUDA device `device`.  Owns scratch memory and
  * device-side bookkeeping; one context may be used from one host thread at a
- * time (calls lock it). */
+ * time (calls lock it).  A call that waits for the device polls for the first
+ * millisecond of each wait, which keeps a core busy, and then sleeps 50 us
+ * between polls. */
 int rt_ctx_create(int device, rt_ctx** out);
 void rt_ctx_destroy(rt_ctx* ctx);
 /* Peel-off (Sect. 2.4) is deferred: each scattering appends one record
@@ -73,8 +75,14 @@ void rt_ctx_destroy(rt_ctx* ctx);
  * kernel marches every (record, observer) pair after the tracer.  The queue
  * holds min(max_records, 2 x packages of the launch) records (at least 2^20);
  * scatterings beyond it peel off inline in the tracer, with the same
- * results.  max_records = 0 disables deferral, < 0 restores the default
- * (2^27).  Takes effect at the next launch (and at rt_batch_create). */
+ * results.  Before the second kernel the records are sorted into a second
+ * buffer: of the queue's capacity up to 2^22 records (50 to 200 MB in FP32, 84
+ * to 336 MB in FP64, and 4 B per record of keys), beyond that of the records
+ * there are.  Without room for it they are marched unsorted, with the same
+ * results.  Both buffers stay with the context until it is destroyed.
+ * max_records = 0 disables deferral, < 0 restores the default (2^27).  Takes
+ * effect at the next launch (and at rt_batch_create; captured batches are not
+ * sorted). */
 int rt_ctx_set_peel_queue(rt_ctx* ctx, int64_t max_records);
 /* Tiled tracing (the GPU form of the grid-by-grid processing of Sect. 2.2 and
  * App. A): for single-job rt_trace / rt_peel / rt_lambda_iterate launches the
@@ -417,7 +425,9 @@ int rt_tune_load(rt_ctx* ctx, const char* path);
  * that runs alone); requests arriving meanwhile join the next launch of
  * whichever slot frees first, so the slots' work overlaps on the device.
  * Results stay on the device (counted in the budget) until
- * rt_server_fetch. */
+ * rt_server_fetch.  Each slot's context keeps its own scratch (job tables,
+ * peel-off queue and its sort buffer: rt_ctx_set_peel_queue), which hbm_budget
+ * does not count. */
 typedef struct {
   size_t hbm_budget;
   int max_slots;          /* 1..16 */

@@ -267,8 +267,8 @@ static PeelQueue make_queue(DevBuf& buf, long long max_records, bool peel, int n
 
 // wait for an event with a deadline; the device keeps running on timeout.
 // The first millisecond is polled (a small call's work takes 0.1 to 1 ms, and
-// a sleep of 50 us ends up to 100 us late), then the thread sleeps between
-// polls.
+// a sleep of 50 us ends up to 100 us late), which keeps the calling thread's
+// core busy that long, then the thread sleeps between polls.
 static int wait_event(cudaEvent_t ev, double timeout_s) {
   const auto t0 = std::chrono::steady_clock::now();
   for (;;) {
@@ -1106,8 +1106,13 @@ static int make_cfg(rt_ctx* c, int precision, bool peel, const rt_trace_params* 
 // for 4e7; the 9.2e6-cell disc (a few MB) 159 against 165 ms for 1e8.  With
 // few packages per bin every (bin, tile) pair of a round brings its cells
 // from DRAM for a handful of crossings: tiles need a package per bin for
-// every 48 counted cells.  The FP64 tracer is bound by the FP64 pipe either
-// way; it takes tiles where the whole grid exceeds one tile's 48 MB.
+// every 48 counted cells.  FP64 launches take tiles where the whole grid
+// exceeds one tile's 48 MB, a line from before their untiled tracer went down
+// to the leaf in a pass, and no longer the faster side of it: untiled against
+// tiled (4 wavelengths) 5.6 against 15.6 ms for 2e5 and 62 against 77 ms for
+// 4e6 packages on a cloud of 4.5e6 cells, 6.3 / 24.5 and 66 / 117 ms on the deep
+// cloud of 9.4e6, 9.8 / 26.0 and 105 / 132 ms on one of 2.4e7
+// (rt_ctx_set_tiles(ctx, 0) turns them off).
 // The tiles' edge: 2^tsh root cells, each tile's words and accumulators at
 // most 48 MB.
 static bool choose_tiles(const rt_ctx* c, const rt_grid* G, int n_jobs, int precision, int n_lambda, long long total,
@@ -1216,8 +1221,13 @@ static int run_tiled(rt_ctx* c, TileRun T, int n_lambda, int precision, bool pee
 // records are counting-sorted into a second buffer.  A queue of at most
 // RT_PEEL_SORT_BLIND records gets a second buffer of its whole capacity and
 // its length stays on the device: reading it back would leave the GPU idle
-// for the wait and the launches behind it.  For a longer queue that wait is
-// small beside the march, and the buffer takes only the records there are.
+// for the wait and the launches behind it.  Sort and march, length on the
+// device against read back: 38 / 53 us (700 records, one map), 86 / 103 us (640,
+// six maps), 191 / 208 us (6.8e4), 317 / 355 us (1.4e5), 527 / 570 us (2.7e5);
+// the whole call 5 to 16 us less while it takes under a millisecond.  The line
+// bounds the second buffer, 200 MB of FP32 records (336 MB in FP64): a longer
+// queue's wait is small beside its march, and its buffer takes only the
+// records there are.
 #ifndef RT_PEEL_SORT
 #define RT_PEEL_SORT 1
 #endif

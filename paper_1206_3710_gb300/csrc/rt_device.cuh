@@ -91,8 +91,8 @@ struct Num<double> {
   static __device__ __forceinline__ double log_(double x) { return log(x); }
   static __device__ __forceinline__ double expm1_(double x) { return expm1(x); }
   // q = 1 - exp(-x), e = 1 - q: Taylor series below 1/8 (relative remainder
-  // below 3e-17 with the terms to x^10, below 2^-9 with those to x^5), exp
-  // above
+  // below 3e-17 with the terms to x^10; below 2^-9 with those to x^5, 4e-17),
+  // exp above
   static __device__ __forceinline__ void absorb_pair(double x, double& q, double& e) {
     const int hi = __double2hiint(x);
     if (hi < 0x3FC00000) {
@@ -179,9 +179,10 @@ struct Geo {
 };
 
 // The next node to visit: `pending` is an array index whose node sits at
-// level k on the path to the package's leaf.  Every loop iteration loads
-// exactly one node word; a refined node advances one level, a leaf ends the
-// search.  Lanes therefore never wait on another lane's multi-level descent.
+// level k on the path to the package's leaf.  A refined node's word advances
+// one level, a leaf's ends the search.  Most loops load one word an iteration,
+// so that no lane waits for another's descent; the kernels whose form says so
+// (PATH_LEAF) go down to the leaf within a pass.
 struct Cursor {
   uint32_t pending;
   int k;

@@ -7,12 +7,13 @@
 // clock against 128 for 32-bit integers: the emission of 2.8e8 (cell, bin)
 // pairs took 26.6 ms, all of it on the FP64 pipe.  Here every step works on
 // 64-bit fixed-point numbers (products by 32 x 32 -> 64 multiply-adds):
-//   z = x log2 e, 2^-z = 2^-k 2^-f, 2^-f = T_j e^-r with j the leading 8 bits
+//   z = x log2 e, 2^-z = 2^-k 2^-f, 2^-f = T_j e^-r with j the leading 9 bits
 //   of f (the table-driven exponential of Tang, ACM TOMS 15, 1989, and, for
 //   1 - 2^-f at small z, TOMS 18, 1992), e^-r by its Taylor series,
 //   1 / (e^x - 1) = 2^-z / (1 - 2^-z), the reciprocal by Newton's iteration.
-// Fixed point keeps about 2^-62, so the error of a term (against 64 bits and
-// more) is that of its rounded inputs h nu and k T, as before.
+// Fixed point keeps about 2^-62 (the reciprocal 2^-57 for arguments within
+// 2^-57 of a power of two, 2^-59 otherwise), so the error of a term (against 64
+// bits and more) is that of its rounded inputs h nu and k T, as before.
 #pragma once
 
 #include <stdint.h>
@@ -74,7 +75,9 @@ RT_HD Norm64 norm64(double v) {
   return r;
 }
 
-// about 2^127 / d for d in [2^63, 2^64): relative error below 2^-60
+// about 2^127 / d for d in [2^63, 2^64): relative error below 2^-59 (2e8 random
+// arguments and the neighbours of powers of two: 2^-59.5), for d below 2^63 + 64,
+// where the quotient is held at 2^64 - 1, below 2^-57
 RT_HD uint64_t recip64(uint64_t d) {
   const uint32_t dh = (uint32_t)(d >> 32), dl = (uint32_t)d;
   // seed to about 2^-21, held below 2^32
@@ -89,7 +92,8 @@ RT_HD uint64_t recip64(uint64_t d) {
   const int32_t eh = (int32_t)(e >> 21);
   const int64_t es = e + (((int64_t)eh * eh) >> 21);
   const int64_t c = (((es >> 16) * (int64_t)y0) >> 15) + (int64_t)(((es & 0xFFFF) * (uint64_t)y0) >> 31);
-  // at d = 2^63 the quotient is 2^64: held below it
+  // at d = 2^63 the quotient is 2^64, and the iteration may reach that a
+  // little above: held below it
   return d < 0x8000000000000040ull ? ~0ull : ((uint64_t)y0 << 32) + (uint64_t)c;
 }
 

@@ -592,11 +592,21 @@ struct MaxThreads {
 // pass, and takes its segment with the others, or one level per pass.  The
 // first keeps more lanes at the segment, but the warp waits for the deepest
 // descent: it pays where descents are frequent (the grids with a stored
-// path) and short.  Tracer and marches, one level against down to the leaf:
-// deep cloud (3 levels) 6.26 / 5.86 ms, discs of 6 and 8 levels 4.77 / 4.62 and
-// 12.2 / 11.8 ms, but of 10 levels (9.2e6 cells) 14.6 / 15.2 ms; FP64, which
-// waits for its pipe anyway, 3.37 / 2.70 ms.  Without a stored path (128^3
-// cloud) 5.23 / 5.63 ms.
+// path) and short.  One level a pass / down to the leaf, each a kernel of its
+// own, in ms:
+//                              star's packages  dust packages  3 oblique maps
+//   deep cloud, 3 levels       3.03 / 2.75 (field)             3.02 / 2.90
+//   disc,  6 levels, 2.7e4     0.90 / 0.77      5.70 / 5.88    0.92 / 0.90
+//   disc,  8 levels, 5.7e5     1.24 / 1.11      5.17 / 5.32    1.11 / 1.11
+//   disc,  9 levels, 1.1e6     1.29 / 1.14      5.33 / 5.45    1.15 / 1.17
+//   disc, 10 levels, 3.1e6     1.44 / 1.30      5.57 / 5.63    1.09 / 1.18
+//   disc, 10 levels, 9.2e6     1.78 / 1.65      5.12 / 5.30    1.33 / 1.48
+//   disc, 12 levels, 8.9e6     1.67 / 1.51      7.33 / 7.44    1.10 / 1.30
+// The tracer gains at every depth but for dust packages, whose lives are a few
+// passes; the marches lose from 10 levels on, and the line lies where they
+// begin to.  (Dust packages would have the other form at any depth, a star's
+// this one.)  FP64, which waits for its pipe anyway: 3.37 / 2.70 ms (32^3 clump
+// with a map).  Without a stored path (128^3 cloud) 5.23 / 5.63 ms.
 // A kernel of its own for each (PATH): deciding it at run time cost the
 // 9.2e6-cell disc 6 %.
 enum { PATH_NONE = 0, PATH_LEVEL = 1, PATH_LEAF = 2 };
@@ -1013,11 +1023,11 @@ __global__ void __launch_bounds__(MaxThreads<R, MODE>::value, MinBlocks<R, MODE>
 
     // ------------------------------------------------------------- fast path
     // Step cells until ev_batch lanes of the warp have met an event, or
-    // none steps any more.  One node word per lane and pass: a refined node
-    // advances the descent by a level, a leaf gets one segment (Sect. 2.3)
-    // and a face crossing.  The word of the next node is fetched as soon as
-    // the crossing has named it, so the segment's absorption and deposit run
-    // while the load is under way.
+    // none steps any more.  A leaf gets one segment (Sect. 2.3) and a face
+    // crossing; a refined node advances the descent by a level, which takes
+    // the lane's pass, or down to the leaf within the pass (PATH_LEAF).  The
+    // word of the next node is fetched as soon as the crossing has named it,
+    // so the segment's absorption and deposit run while the load is under way.
     int ev = (st == ST_TRACE || st == ST_PEEL) ? EV_NONE : EV_IDLE;
     // one pass of the loop; a warp none of whose lanes marches an inline
     // peel-off (the deferred queue had room) runs the tracing-only form
